@@ -7,15 +7,15 @@
 // phase 2 takes each deviation vector through the twelve stages of the linear
 // variational equation w' = J_s w with those Hessians.  The vectors never act
 // on the orbit, so this is DOP853 on the joint system (x, w_1..w_k, M_p), and an
-// adaptive trial that is rejected costs only phase 1.  Stage derivatives and
-// Hessians live in a per-thread column of shared memory, not in registers: on
-// GB300 a warp's FP64 FMA occupies its sub-partition's FP64 unit for 64 cycles
-// while a 64-bit shared-memory access costs about 2 cycles of the SM's shared-
-// memory bandwidth, so the stage traffic is cheap next to the arithmetic and
-// the registers stay free of the up to nine live stages of each phase.  The LD
-// integrand is evaluated only at the eight stages with b_s != 0 (the LD never
-// feeds back into a stage).  Every coefficient is a compile-time constant: the
-// zero entries of the tableau generate no instructions.
+// adaptive trial that is rejected costs only phase 1.  Both phases run the
+// pair in Nystrom form (below), which needs one stage sum per degree of freedom
+// instead of two.  The stage Hessians live in a per-thread column of shared
+// memory: on GB300 a warp's FP64 FMA occupies its sub-partition's FP64 unit for
+// 64 cycles while a 64-bit shared-memory access costs about 2 cycles of the SM's
+// shared-memory bandwidth, so re-reading them for every vector is cheap next to
+// the arithmetic.  The LD integrand is evaluated only at the eight stages with
+// b_s != 0 (the LD never feeds back into a stage).  Every coefficient is a
+// compile-time constant: the zero entries generate no instructions.
 #pragma once
 
 #include <math.h>
@@ -91,74 +91,119 @@ __device__ __forceinline__ void static_for(F&& f)
     }
 }
 
-// True when a later stage reads stage j.
-constexpr bool read_later(int j)
+// The pair in Nystrom form.  Every system here is q' = p, p' = F(q), and its
+// variational equation u' = v, v' = -H(q) u, so a stage's momentum derivative
+// depends on the stage's position alone and the position derivatives p_s can be
+// eliminated: with G_s = h^2 F(q_s),
+//   q_s = q + c_s h p + sum_k abar_sk G_k,         abar = A A,  c_s = sum_j a_sj,
+//   q'  = q + h p + sum_k bbar_k G_k,              bbar = b A,
+//   p'  = p + (1/h) sum_s b_s G_s,
+// the same step in exact arithmetic (Hairer, Norsett and Wanner, Sec. II.14)
+// with one sum per degree of freedom and stage instead of two.  The products
+// are formed here in double-double arithmetic from the tableau above, so each
+// coefficient is the correctly rounded one; the pair's order conditions make
+// some of them vanish (abar_s1 for s >= 5, bbar_1..4, bbar_11), which leaves
+// rounding residues of the decimal tableau below 1e-13 that are set to zero.
+struct Dd {
+    double hi, lo;
+};
+constexpr Dd dd_add_prod(Dd s, double a, double b)
 {
-    for (int s = j + 1; s < 12; ++s)
-        if (kA[s][j] != 0.0) return true;
-    return false;
+    // exact product a b = p + e (Veltkamp splitting, Dekker's product)
+    const double ca = 134217729.0 * a, ah = ca - (ca - a), al = a - ah;
+    const double cb = 134217729.0 * b, bh = cb - (cb - b), bl = b - bh;
+    const double p = a * b, e = ((ah * bh - p) + ah * bl + al * bh) + al * bl;
+    // s + (p + e): Knuth's two-sum of the high parts, then renormalise
+    const double t = s.hi + p, bb = t - s.hi, err = (s.hi - (t - bb)) + (p - bb);
+    const double lo = err + s.lo + e, hi = t + lo;
+    return Dd{hi, lo - (hi - t)};
 }
-template <int J>
-constexpr bool kReadLater = read_later(J);
-static_assert(!read_later(11), "the last stage is never read by another stage");
-
-// The last stage that reads stage j's derivative (-1: none).
-constexpr int last_reader(int j)
+constexpr double dd_value(Dd s)
 {
-    int r = -1;
-    for (int s = j + 1; s < 12; ++s)
-        if (kA[s][j] != 0.0) r = s;
-    return r;
+    return (s.hi < 1e-13 && s.hi > -1e-13) ? 0.0 : s.hi;
 }
-
-// Slab row of stage s's derivative: the lowest row whose occupant no stage
-// after s reads (a stage reads all of its inputs before it writes its own
-// derivative, so a row read last by stage s itself can take it); -1 for a
-// stage that no later stage reads.  Stages 2 and 3 of the pair are read only
-// up to stages 3 and 5, so 11 derivatives fit in 9 rows.
-constexpr int k_row(int s)
+struct Nystrom {
+    double a[12][12], c[12], b[12], e5[12], e3[12];
+};
+constexpr Nystrom make_nystrom()
 {
-    int occ[12] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
-    for (int t = 0; t <= s; ++t) {
-        if (!read_later(t)) {
-            if (t == s) return -1;
-            continue;
+    Nystrom n{};
+    for (int k = 0; k < 12; ++k) {
+        Dd sb{0, 0}, s5{0, 0}, s3{0, 0}, sc{0, 0};
+        for (int j = 0; j < 12; ++j) {
+            sc = dd_add_prod(sc, kA[k][j], 1.0);
+            sb = dd_add_prod(sb, kB[j], kA[j][k]);
+            s5 = dd_add_prod(s5, kE5[j], kA[j][k]);
+            s3 = dd_add_prod(dd_add_prod(s3, kB[j], kA[j][k]), -kB3[j], kA[j][k]);
         }
-        int row = 0;
-        while (occ[row] >= 0 && last_reader(occ[row]) > t) ++row;
-        occ[row] = t;
-        if (t == s) return row;
+        n.c[k] = sc.hi;
+        n.b[k] = dd_value(sb);
+        n.e5[k] = dd_value(s5);
+        n.e3[k] = dd_value(s3);
+        for (int s = 0; s < 12; ++s) {
+            Dd sa{0, 0};
+            for (int j = 0; j < 12; ++j) sa = dd_add_prod(sa, kA[s][j], kA[j][k]);
+            n.a[s][k] = dd_value(sa);
+        }
     }
-    return -1;
+    return n;
 }
-constexpr int k_rows()
+constexpr Nystrom kNys = make_nystrom();
+constexpr int nys_terms()
 {
     int n = 0;
     for (int s = 0; s < 12; ++s)
-        if (k_row(s) + 1 > n) n = k_row(s) + 1;
+        for (int k = 0; k < 12; ++k) n += kNys.a[s][k] != 0.0;
     return n;
 }
+template <int S, int K>
+constexpr double kNa = kNys.a[S][K];
 template <int S>
-constexpr int kRow = k_row(S);
-static_assert(k_rows() == 9, "the DOP853 pair's derivatives fit in 9 rows");
+constexpr double kNc = kNys.c[S];
+template <int S>
+constexpr double kNb = kNys.b[S];
+template <int S>
+constexpr double kN5 = kNys.e5[S];
+template <int S>
+constexpr double kN3 = kNys.e3[S];
+static_assert(nys_terms() == 48, "the vanishing products of the pair are recognised");
 
-// A thread's column of the block's shared array: H[s][t] (stage Hessians,
-// packed upper triangle, 12 stages) then the stage derivatives a later stage
-// reads, in the k_rows() rows given by k_row, entry e at base[e * kBlock].
-// Accesses are volatile so that stage values are re-read from shared memory
-// instead of being kept in registers.
+// sum_{j<S} abar_Sj G_j[i] added to acc.
+template <int S, int N>
+__device__ __forceinline__ double nys_sum(double acc, const double (*G)[N], const int i)
+{
+    static_for<0, S>([&](auto jc) {
+        constexpr int j = decltype(jc)::value;
+        constexpr double c = kNa<S, j>;
+        if constexpr (c != 0.0) acc = fma(c, G[j][i], acc);
+    });
+    return acc;
+}
+
+// Constants of a step of size h.  Steps too small for 1/h (a first guess far
+// below the rounding of the state) leave the momenta as they are.
+struct StepH {
+    double h, nh2, rh;  // h, -h^2, 1/h
+};
+__device__ __forceinline__ StepH step_h(const double h)
+{
+    return StepH{h, -h * h, fabs(h) > 1e-290 ? 1.0 / h : 0.0};
+}
+
+// A thread's column of the block's shared array: -h^2 Hess V of the twelve
+// stages (packed upper triangle), then the orbit's deviation vectors, entry e
+// at base[e * kBlock].  The vectors are worked one after another in a loop that
+// is not unrolled: held in registers they and the unrolled loop took 255
+// registers with spills at k = 4, and the code did not fit the instruction
+// cache.  Accesses are volatile so that the Hessians are re-read by each vector
+// instead of being kept in registers; the stage values G_s of the vector in
+// hand (at most ten live, N doubles each) stay in registers.
 template <class Sys>
 struct Slab {
     static constexpr int D = 2 * Sys::N, NH = Sys::NH;
-    static constexpr int kDoubles = 12 * NH + k_rows() * D;
     volatile double* base;
     __device__ __forceinline__ volatile double& H(int s, int t) const { return base[(s * NH + t) * kBlock]; }
-    template <int S>
-    __device__ __forceinline__ volatile double& K(int i) const
-    {
-        static_assert(kRow<S> >= 0, "a stage derivative that no later stage reads is not stored");
-        return base[(12 * NH + kRow<S> * D + i) * kBlock];
-    }
+    __device__ __forceinline__ volatile double& W(int j, int c) const { return base[(12 * NH + j * D + c) * kBlock]; }
 };
 
 template <class Sys>
@@ -168,141 +213,156 @@ __device__ __forceinline__ Slab<Sys> my_slab()
     return Slab<Sys>{dsm + threadIdx.x};
 }
 
-template <class Sys>
+// Shared bytes of a block whose threads keep K deviation vectors in the slab.
+template <class Sys, int K>
 constexpr size_t slab_bytes()
 {
-    return (size_t)Slab<Sys>::kDoubles * kBlock * sizeof(double);
+    return (size_t)(12 * Sys::NH + K * 2 * Sys::N) * kBlock * sizeof(double);
 }
 
-// sum_{j<S} a_Sj K_j[i] over the nonzero a_Sj (0 for S = 0).
-template <int S, class Sys>
-__device__ __forceinline__ double stage_sum(const Slab<Sys>& sl, const int i)
-{
-    double acc = 0.0;
-    static_for<0, S>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        constexpr double c = kA[S][j];
-        if constexpr (c != 0.0) acc = fma(c, sl.template K<j>(i), acc);
-    });
-    return acc;
-}
-
-// Phase 1, the orbit's twelve stages from x with step h:
-//   K_s = f(x + h sum_{j<s} a_sj K_j),   xn = x + h sum_s b_s K_s,
-//   dL = |h| sum_s b_s g(K_s)  (g the LD integrand; the LD grows with |t|),
-// the stage Hessians into the slab, and with ERR the error sums
-// err5_i = sum_s e5_s K_s,i and err3_i = sum_s (b_s - b3_s) K_s,i.
+// Phase 1, the orbit's twelve stages from x = (q, p) in Nystrom form:
+//   xn = the step's end point,
+//   dL = |h| sum_s b_s g_s  (g the LD integrand of f_s = (p_s, F_s); the LD grows
+//        with |t|), with h p_s = h p + sum_j a_sj G_j formed only at the stages
+//        with b_s != 0,
+// the stage matrices -h^2 Hess V into the slab, and with ERR the error sums
+// times h: h err5_q = sum_k (e5 A)_k G_k, h err5_p = (1/h) sum_s e5_s G_s, and err3
+// likewise.  The small terms are summed first and added to the state last.
 template <class Sys, bool LD, bool ERR>
-__device__ __forceinline__ void orbit_step(const Slab<Sys>& sl, const double* x, const double h,
+__device__ __forceinline__ void orbit_step(const Slab<Sys>& sl, const double* x, const StepH sh,
                                            const int ld_sqrt, const double ld_p, const SysPar& sp,
                                            double* xn, double& dL, double* e5, double* e3)
 {
-    constexpr int D = 2 * Sys::N, NH = Sys::NH;
-    double sb[D], s5[D], s3[D];
-    double sL = 0.0;
+    constexpr int N = Sys::N, NH = Sys::NH;
+    double G[12][N], hp[N], sq[N], sv[N], q5[N], q3[N], p5[N], p3[N];
+    double sL = 0.0, sLq = 0.0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        hp[i] = sh.h * x[N + i];
+        sq[i] = sv[i] = q5[i] = q3[i] = p5[i] = p3[i] = 0.0;
+    }
     static_for<0, 12>([&](auto sc) {
         constexpr int s = decltype(sc)::value;
-        double xs[D], f[D], H[NH];
+        double qs[N], H[NH];
 #pragma unroll
-        for (int i = 0; i < D; ++i) xs[i] = (s == 0) ? x[i] : fma(h, stage_sum<s>(sl, i), x[i]);
-        Sys::eval(xs, f, H, sp);
+        for (int i = 0; i < N; ++i)
+            qs[i] = (s == 0) ? x[i] : nys_sum<s, N>(fma(kNc<s>, hp[i], x[i]), G, i);
+        Sys::eval_scaled(qs, sh.nh2, G[s], H, sp);
 #pragma unroll
         for (int t = 0; t < NH; ++t) sl.H(s, t) = H[t];
-        if constexpr (kReadLater<s>) {
+        constexpr double cb = kB[s], nb = kNb<s>;
 #pragma unroll
-            for (int i = 0; i < D; ++i) sl.template K<s>(i) = f[i];
-        }
-        constexpr double cb = kB[s], c5 = kE5[s], c3 = kB[s] - kB3[s];
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            if constexpr (s == 0) {
-                sb[i] = cb * f[i];
-                if constexpr (ERR) {
-                    s5[i] = c5 * f[i];
-                    s3[i] = c3 * f[i];
-                }
-            } else {
-                if constexpr (cb != 0.0) sb[i] = fma(cb, f[i], sb[i]);
-                if constexpr (ERR && c5 != 0.0) s5[i] = fma(c5, f[i], s5[i]);
-                if constexpr (ERR && c3 != 0.0) s3[i] = fma(c3, f[i], s3[i]);
+        for (int i = 0; i < N; ++i) {
+            if constexpr (nb != 0.0) sq[i] = fma(nb, G[s][i], sq[i]);
+            if constexpr (cb != 0.0) sv[i] = fma(cb, G[s][i], sv[i]);
+            if constexpr (ERR) {
+                if constexpr (kN5<s> != 0.0) q5[i] = fma(kN5<s>, G[s][i], q5[i]);
+                if constexpr (kN3<s> != 0.0) q3[i] = fma(kN3<s>, G[s][i], q3[i]);
+                constexpr double c5 = kE5[s], c3 = kB[s] - kB3[s];
+                if constexpr (c5 != 0.0) p5[i] = fma(c5, G[s][i], p5[i]);
+                if constexpr (c3 != 0.0) p3[i] = fma(c3, G[s][i], p3[i]);
             }
         }
         if constexpr (LD && cb != 0.0) {
-            // p = 1/2: the stage's sum of square roots in double-float, widened once
-            const double g = ld_sqrt ? ff_to_f64(ff_sum_sqrt_abs<D>(f)) : ld_integrand_pow<D>(f, ld_p);
-            sL = fma(cb, g, sL);
+            double hps[N];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                hps[i] = hp[i];
+                static_for<0, s>([&](auto jc) {
+                    constexpr int j = decltype(jc)::value;
+                    constexpr double c = kA[s][j];
+                    if constexpr (c != 0.0) hps[i] = fma(c, G[j][i], hps[i]);
+                });
+            }
+            if (ld_sqrt) {
+                // p = 1/2: sums of sqrt|h p_s| and of sqrt|h^2 F_s| in double-float, widened once;
+                // their factors |h|^(-1/2) and 1/|h| are applied at the end of the step
+                sLq = fma(cb, ff_to_f64(ff_sum_sqrt_abs<N>(hps)), sLq);
+                sL = fma(cb, ff_to_f64(ff_sum_sqrt_abs<N>(G[s])), sL);
+            } else {
+                double f[2 * N];
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    f[i] = sh.rh * hps[i];
+                    f[N + i] = sh.rh * (sh.rh * G[s][i]);
+                }
+                sL = fma(cb, ld_integrand_pow<2 * N>(f, ld_p), sL);
+            }
         }
     });
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-        xn[i] = fma(h, sb[i], x[i]);
+    for (int i = 0; i < N; ++i) {
+        xn[i] = x[i] + (hp[i] + sq[i]);
+        xn[N + i] = fma(sh.rh, sv[i], x[N + i]);
         if constexpr (ERR) {
-            e5[i] = s5[i];
-            e3[i] = s3[i];
+            e5[i] = q5[i];
+            e3[i] = q3[i];
+            e5[N + i] = sh.rh * p5[i];
+            e3[N + i] = sh.rh * p3[i];
         }
     }
-    if constexpr (LD) dL = fabs(h) * sL;
+    if constexpr (LD) dL = ld_sqrt ? fma(sqrt(fabs(sh.h)), sLq, sL) : fabs(sh.h) * sL;
 }
 
-// Phase 2, one deviation vector w = (dq, dp) through the twelve stages of
-// w' = J_s w, J_s w = (dp, -H_s dq), with the Hessians of phase 1:
-//   M_s = J_s (w + h sum_{j<s} a_sj M_j),   w <- w + h sum_s b_s M_s.
-// The stage derivatives M_s reuse the slab's K rows.
+// Phase 2, one deviation vector w = (u, v) through the twelve stages of
+// u' = v, v' = -H_s u in Nystrom form with the matrices of phase 1:
+// G_s = -h^2 H_s u_s.  204 FP64 instructions for 2 DOF (328 with the stage sums
+// of u and v kept apart): the 256 x 256 Henon-Heiles grid with k = 4 and the LD, 60
+// steps, took 16.3 ms so and takes 10.6 ms.
 template <class Sys>
-__device__ __forceinline__ void vector_step(const Slab<Sys>& sl, double* w, const double h)
+__device__ __forceinline__ void vector_step(const Slab<Sys>& sl, double* w, const StepH sh)
 {
-    constexpr int N = Sys::N, D = 2 * N, NH = Sys::NH;
-    double sb[D];
+    constexpr int N = Sys::N, NH = Sys::NH;
+    double G[12][N], hv[N], sq[N], sv[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        hv[i] = sh.h * w[N + i];
+        sq[i] = sv[i] = 0.0;
+    }
     static_for<0, 12>([&](auto sc) {
         constexpr int s = decltype(sc)::value;
-        double ws[D], m[D], H[NH];
+        double us[N], H[NH];
 #pragma unroll
-        for (int i = 0; i < D; ++i) ws[i] = (s == 0) ? w[i] : fma(h, stage_sum<s>(sl, i), w[i]);
+        for (int i = 0; i < N; ++i)
+            us[i] = (s == 0) ? w[i] : nys_sum<s, N>(fma(kNc<s>, hv[i], w[i]), G, i);
 #pragma unroll
         for (int t = 0; t < NH; ++t) H[t] = sl.H(s, t);
+        constexpr double cb = kB[s], nb = kNb<s>;
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-            m[i] = ws[N + i];
-            double acc = H[hidx<N>(i, 0)] * ws[0];
+            double acc = H[hidx<N>(i, 0)] * us[0];
 #pragma unroll
-            for (int q = 1; q < N; ++q) acc = fma(H[hidx<N>(i, q)], ws[q], acc);
-            m[N + i] = -acc;
-        }
-        if constexpr (kReadLater<s>) {
-#pragma unroll
-            for (int i = 0; i < D; ++i) sl.template K<s>(i) = m[i];
-        }
-        constexpr double cb = kB[s];
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-            if constexpr (s == 0)
-                sb[i] = cb * m[i];
-            else if constexpr (cb != 0.0)
-                sb[i] = fma(cb, m[i], sb[i]);
+            for (int m = 1; m < N; ++m) acc = fma(H[hidx<N>(i, m)], us[m], acc);
+            G[s][i] = acc;
+            if constexpr (nb != 0.0) sq[i] = fma(nb, acc, sq[i]);
+            if constexpr (cb != 0.0) sv[i] = fma(cb, acc, sv[i]);
         }
     });
 #pragma unroll
-    for (int i = 0; i < D; ++i) w[i] = fma(h, sb[i], w[i]);
+    for (int i = 0; i < N; ++i) {
+        w[i] = w[i] + (hv[i] + sq[i]);
+        w[N + i] = fma(sh.rh, sv[i], w[N + i]);
+    }
 }
 
 // Error norm of a trial over the orbit components:
 //   scale_i = atol + rtol max(|x_i|, |xn_i|),  E5 = sum (err5_i / scale_i)^2,
-//   E3 likewise, err = |h| E5 / sqrt(D (E5 + 0.01 E3)) (0 when both vanish).
+//   E3 likewise, err = |h| E5 / sqrt(D (E5 + 0.01 E3)) (0 when both vanish);
+// e5 and e3 are h err5 and h err3, which absorbs the factor |h|.
 template <int D>
 __device__ __forceinline__ double err_norm(const double* x, const double* xn, const double* e5,
-                                           const double* e3, const double h, const double atol,
-                                           const double rtol)
+                                           const double* e3, const double atol, const double rtol)
 {
     double E5 = 0.0, E3 = 0.0;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        const double sc = atol + rtol * fmax(fabs(x[i]), fabs(xn[i]));
-        const double q5 = e5[i] / sc, q3 = e3[i] / sc;
+        const double rsc = 1.0 / (atol + rtol * fmax(fabs(x[i]), fabs(xn[i])));
+        const double q5 = e5[i] * rsc, q3 = e3[i] * rsc;
         E5 = fma(q5, q5, E5);
         E3 = fma(q3, q3, E3);
     }
     if (E5 == 0.0 && E3 == 0.0) return 0.0;
-    return fabs(h) * E5 / sqrt((double)D * (E5 + 0.01 * E3));
+    return E5 / sqrt((double)D * (E5 + 0.01 * E3));
 }
 
 // SALI of two vectors (each normalised first): min(|u + v|, |u - v|).
@@ -326,26 +386,39 @@ __device__ __forceinline__ double sali2(const double* a, const double* b)
     return sqrt(fmin(sp, sm));
 }
 
-// What follows every completed step (the chs_integrate_batch contract):
-// renormalisation, escape, and at health checks finiteness, energy drift and
-// the early exit.  Returns the orbit status.
+// The K deviation vectors of the slab through one step, scaled to unit length
+// with renorm.
 template <class Sys, int K>
-__device__ __forceinline__ int32_t post_step(const double* x, double (*w)[2 * Sys::N],
-                                             const double L, const StepArgs& a, const SysPar& sp,
-                                             const bool check, const double h0, double& dhm)
+__device__ __forceinline__ void vectors_step(const Slab<Sys>& sl, const StepH sh, const int renorm)
+{
+    constexpr int D = 2 * Sys::N;
+#pragma unroll 1
+    for (int j = 0; j < K; ++j) {
+        double w[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) w[c] = sl.W(j, c);
+        vector_step<Sys>(sl, w, sh);
+        double inv = 1.0;
+        if (renorm) {
+            double n2 = w[0] * w[0];
+#pragma unroll
+            for (int c = 1; c < D; ++c) n2 = fma(w[c], w[c], n2);
+            inv = rsqrt_ff(n2);
+        }
+#pragma unroll
+        for (int c = 0; c < D; ++c) sl.W(j, c) = w[c] * inv;
+    }
+}
+
+// What follows every completed step and its renormalisation (the
+// chs_integrate_batch contract): escape, and at health checks finiteness,
+// energy drift and the early exit.  Returns the orbit status.
+template <class Sys, int K>
+__device__ __forceinline__ int32_t post_step(const double* x, const Slab<Sys>& sl, const double L,
+                                             const StepArgs& a, const SysPar& sp, const bool check,
+                                             const double h0, double& dhm)
 {
     constexpr int N = Sys::N, D = 2 * N;
-    if (a.renorm) {
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            double n2 = w[j][0] * w[j][0];
-#pragma unroll
-            for (int c = 1; c < D; ++c) n2 = fma(w[j][c], w[j][c], n2);
-            const double inv = rsqrt_ff(n2);
-#pragma unroll
-            for (int c = 0; c < D; ++c) w[j][c] *= inv;
-        }
-    }
     if (a.escape_r2 > 0.0) {
         double r2 = x[0] * x[0];
 #pragma unroll
@@ -356,16 +429,22 @@ __device__ __forceinline__ int32_t post_step(const double* x, double (*w)[2 * Sy
         bool fin = isfinite(L);
 #pragma unroll
         for (int c = 0; c < D; ++c) fin = fin && isfinite(x[c]);
-#pragma unroll
-        for (int j = 0; j < K; ++j)
-#pragma unroll
-            for (int c = 0; c < D; ++c) fin = fin && isfinite(w[j][c]);
+#pragma unroll 1
+        for (int i = 0; i < K * D; ++i) fin = fin && isfinite((double)sl.W(0, i));
         if (!fin) return CHS_ORBIT_NONFINITE;
         const double dH = fabs(Sys::energy(x, sp) - h0);
         dhm = fmax(dhm, dH);
         if (a.dh_limit > 0.0 && dH > a.dh_limit) return CHS_ORBIT_ENERGY_DRIFT;
         if constexpr (K >= 2) {
-            if (a.early_exit && sali2<D>(w[0], w[1]) < a.sali_threshold) return CHS_ORBIT_EARLY_CHAOTIC;
+            if (a.early_exit) {
+                double u[D], v[D];
+#pragma unroll
+                for (int c = 0; c < D; ++c) {
+                    u[c] = sl.W(0, c);
+                    v[c] = sl.W(1, c);
+                }
+                if (sali2<D>(u, v) < a.sali_threshold) return CHS_ORBIT_EARLY_CHAOTIC;
+            }
         }
     }
     return CHS_ORBIT_OK;

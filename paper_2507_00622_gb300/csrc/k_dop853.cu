@@ -37,13 +37,14 @@ k_lyap_small_dp(const StepArgs a, const SysPar sp, const int64_t n, const double
     if (st == CHS_ORBIT_OK && !fin) st = CHS_ORBIT_NONFINITE;
     if (st == CHS_ORBIT_OK) {
         const long long t_start = clock64();
+        const dp::StepH sh = dp::step_h(a.dt);
         int64_t until_qr = a.qr_every;
         int64_t until = a.sample_every > 0 ? a.sample_every : -1;
         for (int64_t s = 1; s <= a.n_steps; ++s) {
             double xn[D], dL = 0.0;
-            dp::orbit_step<Sys, false, false>(sl, x, a.dt, 0, 0.0, sp, xn, dL, nullptr, nullptr);
+            dp::orbit_step<Sys, false, false>(sl, x, sh, 0, 0.0, sp, xn, dL, nullptr, nullptr);
 #pragma unroll
-            for (int j = 0; j < D; ++j) dp::vector_step<Sys>(sl, W[j], a.dt);
+            for (int j = 0; j < D; ++j) dp::vector_step<Sys>(sl, W[j], sh);
 #pragma unroll
             for (int c = 0; c < D; ++c) x[c] = xn[c];
             if (--until_qr == 0 || s == a.n_steps) {
@@ -113,15 +114,15 @@ cudaError_t launch_lyap_small_dp(const SysPar& sp, const StepArgs& a, int64_t n,
     const unsigned g = blocks_for(n, kBlock);
     switch (sp.model) {
     case CHS_HENON_HEILES:
-        k_lyap_small_dp<SysHenonHeiles><<<g, kBlock, dp::slab_bytes<SysHenonHeiles>(), st>>>(
+        k_lyap_small_dp<SysHenonHeiles><<<g, kBlock, dp::slab_bytes<SysHenonHeiles, 0>(), st>>>(
             a, sp, n, ics, ic_status, lambda, status);
         break;
     case CHS_HARMONIC:
-        k_lyap_small_dp<SysHarmonic><<<g, kBlock, dp::slab_bytes<SysHarmonic>(), st>>>(
+        k_lyap_small_dp<SysHarmonic><<<g, kBlock, dp::slab_bytes<SysHarmonic, 0>(), st>>>(
             a, sp, n, ics, ic_status, lambda, status);
         break;
     case CHS_INVERTED:
-        k_lyap_small_dp<SysInverted><<<g, kBlock, dp::slab_bytes<SysInverted>(), st>>>(
+        k_lyap_small_dp<SysInverted><<<g, kBlock, dp::slab_bytes<SysInverted, 0>(), st>>>(
             a, sp, n, ics, ic_status, lambda, status);
         break;
     default:

@@ -15,8 +15,7 @@ __global__ void __launch_bounds__(kBlock)
 k_integrate_adaptive(const StepArgs a, const AdaptArgs ad, const SysPar sp, const EnsPtrs e,
                      const AdaptPtrs ap)
 {
-    constexpr int N = Sys::N, D = 2 * N;
-    constexpr int KK = K > 0 ? K : 1;
+    constexpr int D = 2 * Sys::N;
     const dp::Slab<Sys> sl = dp::my_slab<Sys>();
     const int64_t n = e.n;
     const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -24,13 +23,13 @@ k_integrate_adaptive(const StepArgs a, const AdaptArgs ad, const SysPar sp, cons
     if (e.status[o] != CHS_ORBIT_OK) return;
 
     double* wg = static_cast<double*>(e.w);
-    double x[D], w[KK][D];
+    double x[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) x[c] = e.x[c * n + o];
 #pragma unroll
     for (int j = 0; j < K; ++j)
 #pragma unroll
-        for (int c = 0; c < D; ++c) w[j][c] = wg[(j * D + c) * n + o];
+        for (int c = 0; c < D; ++c) sl.W(j, c) = wg[(j * D + c) * n + o];
     double L = LD ? e.ld[o] : 0.0;
     const double h0 = e.h0[o];
     double dhm = e.dh_max[o];
@@ -50,6 +49,7 @@ k_integrate_adaptive(const StepArgs a, const AdaptArgs ad, const SysPar sp, cons
         if (h < min_step) h = min_step;
         bool rejected = false;
         double xn[D], dL = 0.0, hh = 0.0, err = 0.0;
+        dp::StepH sh{};
         // Each rejection multiplies h by at most 0.9 (0.2 for a non-finite
         // error), so this loop ends once h drops below min_step.
         for (;;) {
@@ -60,9 +60,10 @@ k_integrate_adaptive(const StepArgs a, const AdaptArgs ad, const SysPar sp, cons
             double tn = tt + h;
             if (tn > ad.t_final) tn = ad.t_final;
             hh = tn - tt;
+            sh = dp::step_h(hh);
             double e5[D], e3[D];
-            dp::orbit_step<Sys, LD, true>(sl, x, hh, a.ld_sqrt, a.ld_p, sp, xn, dL, e5, e3);
-            err = dp::err_norm<D>(x, xn, e5, e3, hh, ad.atol, ad.rtol);
+            dp::orbit_step<Sys, LD, true>(sl, x, sh, a.ld_sqrt, a.ld_p, sp, xn, dL, e5, e3);
+            err = dp::err_norm<D>(x, xn, e5, e3, ad.atol, ad.rtol);
             // err^(-1/8) as three square roots and a division
             const double r8 = (err > 0.0) ? 1.0 / sqrt(sqrt(sqrt(err))) : 0.0;
             if (err < 1.0) {
@@ -79,8 +80,7 @@ k_integrate_adaptive(const StepArgs a, const AdaptArgs ad, const SysPar sp, cons
             ++rej;
         }
         if (st != CHS_ORBIT_OK) break;
-#pragma unroll
-        for (int j = 0; j < K; ++j) dp::vector_step<Sys>(sl, w[j], hh);
+        dp::vectors_step<Sys, K>(sl, sh, a.renorm);
 #pragma unroll
         for (int c = 0; c < D; ++c) x[c] = xn[c];
         if (LD) L += dL;
@@ -88,7 +88,7 @@ k_integrate_adaptive(const StepArgs a, const AdaptArgs ad, const SysPar sp, cons
         em = fmax(em, err);
         ++done;
         const bool check = a.sample_every > 0 && (exec0 + done) % a.sample_every == 0;
-        st = dp::post_step<Sys, K>(x, w, L, a, sp, check, h0, dhm);
+        st = dp::post_step<Sys, K>(x, sl, L, a, sp, check, h0, dhm);
         if (check && st == CHS_ORBIT_OK && budget_spent(a, t_start)) st = CHS_ORBIT_STEP_BUDGET;
         if (st != CHS_ORBIT_OK) break;
     }
@@ -98,7 +98,7 @@ k_integrate_adaptive(const StepArgs a, const AdaptArgs ad, const SysPar sp, cons
 #pragma unroll
     for (int j = 0; j < K; ++j)
 #pragma unroll
-        for (int c = 0; c < D; ++c) wg[(j * D + c) * n + o] = w[j][c];
+        for (int c = 0; c < D; ++c) wg[(j * D + c) * n + o] = sl.W(j, c);
     if (LD) e.ld[o] = L;
     e.dh_max[o] = dhm;
     e.n_exec[o] = exec0 + done;
@@ -149,6 +149,7 @@ k_lyap_small_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const 
         if (h < min_step) h = min_step;
         bool rejected = false;
         double xn[D], dL = 0.0, hh = 0.0, tn = tt;
+        dp::StepH sh{};
         // each rejection shrinks h by at least 0.9 (0.2 for a non-finite error)
         for (;;) {
             if (h < min_step) {
@@ -158,9 +159,10 @@ k_lyap_small_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const 
             tn = tt + h;
             if (tn > ad.t_final) tn = ad.t_final;
             hh = tn - tt;
+            sh = dp::step_h(hh);
             double e5[D], e3[D];
-            dp::orbit_step<Sys, false, true>(sl, x, hh, 0, 0.0, sp, xn, dL, e5, e3);
-            const double err = dp::err_norm<D>(x, xn, e5, e3, hh, ad.atol, ad.rtol);
+            dp::orbit_step<Sys, false, true>(sl, x, sh, 0, 0.0, sp, xn, dL, e5, e3);
+            const double err = dp::err_norm<D>(x, xn, e5, e3, ad.atol, ad.rtol);
             const double r8 = (err > 0.0) ? 1.0 / sqrt(sqrt(sqrt(err))) : 0.0;
             if (err < 1.0) {
                 double fac = (err == 0.0) ? 10.0 : fmin(10.0, 0.9 * r8);
@@ -176,7 +178,7 @@ k_lyap_small_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const 
         }
         if (st != CHS_ORBIT_OK) break;
 #pragma unroll
-        for (int j = 0; j < D; ++j) dp::vector_step<Sys>(sl, W[j], hh);
+        for (int j = 0; j < D; ++j) dp::vector_step<Sys>(sl, W[j], sh);
 #pragma unroll
         for (int c = 0; c < D; ++c) x[c] = xn[c];
         tt = tn;
@@ -223,9 +225,9 @@ cudaError_t adapt_sys(int k, bool ld, const StepArgs& a, const AdaptArgs& ad, co
                       const EnsPtrs& e, const AdaptPtrs& ap, cudaStream_t st)
 {
     const unsigned g = blocks_for(e.n, kBlock);
-    constexpr size_t sm = dp::slab_bytes<Sys>();
     return dp::with_k<Sys>(k, [&](auto kc) {
         constexpr int K = decltype(kc)::value;
+        constexpr size_t sm = dp::slab_bytes<Sys, K>();
         if (ld)
             k_integrate_adaptive<Sys, K, true><<<g, kBlock, sm, st>>>(a, ad, sp, e, ap);
         else
@@ -243,15 +245,15 @@ cudaError_t launch_lyap_small_adapt(const SysPar& sp, const StepArgs& a, const A
     const unsigned g = blocks_for(n, kBlock);
     switch (sp.model) {
     case CHS_HENON_HEILES:
-        k_lyap_small_adapt<SysHenonHeiles><<<g, kBlock, dp::slab_bytes<SysHenonHeiles>(), st>>>(
+        k_lyap_small_adapt<SysHenonHeiles><<<g, kBlock, dp::slab_bytes<SysHenonHeiles, 0>(), st>>>(
             a, ad, sp, n, ics, ic_status, lambda, status, n_acc, n_rej);
         break;
     case CHS_HARMONIC:
-        k_lyap_small_adapt<SysHarmonic><<<g, kBlock, dp::slab_bytes<SysHarmonic>(), st>>>(
+        k_lyap_small_adapt<SysHarmonic><<<g, kBlock, dp::slab_bytes<SysHarmonic, 0>(), st>>>(
             a, ad, sp, n, ics, ic_status, lambda, status, n_acc, n_rej);
         break;
     case CHS_INVERTED:
-        k_lyap_small_adapt<SysInverted><<<g, kBlock, dp::slab_bytes<SysInverted>(), st>>>(
+        k_lyap_small_adapt<SysInverted><<<g, kBlock, dp::slab_bytes<SysInverted, 0>(), st>>>(
             a, ad, sp, n, ics, ic_status, lambda, status, n_acc, n_rej);
         break;
     default:

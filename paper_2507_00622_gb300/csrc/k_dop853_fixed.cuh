@@ -14,15 +14,15 @@ using dp::kBlock;
 // steps with the checks of the chs_integrate_batch contract, stored back.
 template <class Sys, int K, bool LD>
 struct DpRun {
-    static constexpr int N = Sys::N, D = 2 * N, KK = K > 0 ? K : 1;
-    double x[D], w[KK][D];
+    static constexpr int N = Sys::N, D = 2 * N;
+    double x[D];
     double L, h0, dhm;
     int64_t exec0, todo, s, until;
     long long t_start;  // clock64 when the orbit was taken up (clock budget)
     int32_t st;
 
     __device__ __forceinline__ void load(const int64_t o, const StepArgs& a, const EnsPtrs& e,
-                                         const dp::Slab<Sys>&)
+                                         const dp::Slab<Sys>& sl)
     {
         const int64_t n = e.n;
         const double* wg = static_cast<const double*>(e.w);
@@ -31,7 +31,7 @@ struct DpRun {
 #pragma unroll
         for (int j = 0; j < K; ++j)
 #pragma unroll
-            for (int c = 0; c < D; ++c) w[j][c] = wg[(j * D + c) * n + o];
+            for (int c = 0; c < D; ++c) sl.W(j, c) = wg[(j * D + c) * n + o];
         L = LD ? e.ld[o] : 0.0;
         h0 = e.h0[o];
         dhm = e.dh_max[o];
@@ -49,9 +49,9 @@ struct DpRun {
     {
         ++s;
         double xn[D], dL = 0.0;
-        dp::orbit_step<Sys, LD, false>(sl, x, a.dt, a.ld_sqrt, a.ld_p, sp, xn, dL, nullptr, nullptr);
-#pragma unroll
-        for (int j = 0; j < K; ++j) dp::vector_step<Sys>(sl, w[j], a.dt);
+        const dp::StepH sh = dp::step_h(a.dt);
+        dp::orbit_step<Sys, LD, false>(sl, x, sh, a.ld_sqrt, a.ld_p, sp, xn, dL, nullptr, nullptr);
+        dp::vectors_step<Sys, K>(sl, sh, a.renorm);
 #pragma unroll
         for (int c = 0; c < D; ++c) x[c] = xn[c];
         if (LD) L += dL;
@@ -60,13 +60,13 @@ struct DpRun {
             until = a.sample_every;
             check = true;
         }
-        st = dp::post_step<Sys, K>(x, w, L, a, sp, check, h0, dhm);
+        st = dp::post_step<Sys, K>(x, sl, L, a, sp, check, h0, dhm);
         if (check && st == CHS_ORBIT_OK && budget_spent(a, t_start)) st = CHS_ORBIT_STEP_BUDGET;
         return st == CHS_ORBIT_OK;
     }
 
     // Writes the orbit back; true when it is still running.
-    __device__ __forceinline__ bool store(const int64_t o, const EnsPtrs& e, const dp::Slab<Sys>&) const
+    __device__ __forceinline__ bool store(const int64_t o, const EnsPtrs& e, const dp::Slab<Sys>& sl) const
     {
         const int64_t n = e.n;
         double* wg = static_cast<double*>(e.w);
@@ -75,7 +75,7 @@ struct DpRun {
 #pragma unroll
         for (int j = 0; j < K; ++j)
 #pragma unroll
-            for (int c = 0; c < D; ++c) wg[(j * D + c) * n + o] = w[j][c];
+            for (int c = 0; c < D; ++c) wg[(j * D + c) * n + o] = sl.W(j, c);
         if (LD) e.ld[o] = L;
         e.dh_max[o] = dhm;
         e.n_exec[o] = exec0 + s;
@@ -128,9 +128,9 @@ cudaError_t fixed_sys(int k, bool ld, const StepArgs& a, const SysPar& sp, const
 {
     const unsigned g = blocks_for(e.n, kBlock);
     const OrbitList l = ol ? *ol : OrbitList{};
-    constexpr size_t sm = dp::slab_bytes<Sys>();
     return dp::with_k<Sys>(k, [&](auto kc) {
         constexpr int K = decltype(kc)::value;
+        constexpr size_t sm = dp::slab_bytes<Sys, K>();
         auto kern = ld ? k_integrate_dp<Sys, K, true> : k_integrate_dp<Sys, K, false>;
         unsigned grid = g;
         if (l.queue) {

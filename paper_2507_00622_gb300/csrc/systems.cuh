@@ -4,6 +4,8 @@
 //   eval(x, f, H)  f = (p, -grad V(q)) (Hamilton's equations) and the packed
 //                  upper triangle H of Hess V(q), which drives the variational
 //                  equations d(dq)/dt = dp, d(dp)/dt = -Hess V(q) dq;
+//   eval_scaled(q, nh2, G, H)  the same for the Nystrom form of DOP853, scaled by
+//                  nh2 = -h^2: G = h^2 F(q) = -h^2 grad V(q) and H = -h^2 Hess V(q);
 //   energy(x)      the Hamiltonian.
 #pragma once
 
@@ -34,6 +36,16 @@ struct SysHenonHeiles {
         f[2] = -q1 * a;
         f[3] = fma(-q1, q1, fma(q2, q2, -q2));
     }
+    __device__ __forceinline__ static void eval_scaled(const double* q, const double nh2, double* G, double* H,
+                                                       const SysPar&)
+    {
+        const double t = nh2 * q[0];
+        H[0] = fma(2.0 * nh2, q[1], nh2);
+        H[1] = t + t;
+        H[2] = fma(-2.0 * nh2, q[1], nh2);
+        G[0] = q[0] * H[0];
+        G[1] = fma(t, q[0], q[1] * fma(-nh2, q[1], nh2));
+    }
     __device__ __forceinline__ static double energy(const double* x, const SysPar&)
     {
         const double q1 = x[0], q2 = x[1];
@@ -55,6 +67,15 @@ struct SysHarmonic {
         f[2] = -x[0];
         f[3] = -x[1];
     }
+    __device__ __forceinline__ static void eval_scaled(const double* q, const double nh2, double* G, double* H,
+                                                       const SysPar&)
+    {
+        H[0] = nh2;
+        H[1] = 0.0;
+        H[2] = nh2;
+        G[0] = nh2 * q[0];
+        G[1] = nh2 * q[1];
+    }
     __device__ __forceinline__ static double energy(const double* x, const SysPar&)
     {
         return 0.5 * (x[2] * x[2] + x[3] * x[3]) + 0.5 * (x[0] * x[0] + x[1] * x[1]);
@@ -73,6 +94,15 @@ struct SysInverted {
         f[1] = x[3];
         f[2] = x[0];
         f[3] = -x[1];
+    }
+    __device__ __forceinline__ static void eval_scaled(const double* q, const double nh2, double* G, double* H,
+                                                       const SysPar&)
+    {
+        H[0] = -nh2;
+        H[1] = 0.0;
+        H[2] = nh2;
+        G[0] = -nh2 * q[0];
+        G[1] = nh2 * q[1];
     }
     __device__ __forceinline__ static double energy(const double* x, const SysPar&)
     {
@@ -105,6 +135,24 @@ struct SysQuartic3 {
         f[3] = -x[0] * d0;
         f[4] = -x[1] * d1;
         f[5] = -x[2] * d2;
+    }
+    __device__ __forceinline__ static void eval_scaled(const double* q, const double nh2, double* G, double* H,
+                                                       const SysPar& sp)
+    {
+        const double e2 = 2.0 * sp.eps * nh2, e4 = 4.0 * sp.eps * nh2;
+        const double s0 = q[0] * q[0], s1 = q[1] * q[1], s2 = q[2] * q[2], e40 = e4 * q[0];
+        const double d0 = fma(e2, s1 + s2, nh2);
+        const double d1 = fma(e2, s0 + s2, nh2);
+        const double d2 = fma(e2, s0 + s1, nh2);
+        H[hidx<3>(0, 0)] = d0;
+        H[hidx<3>(1, 1)] = d1;
+        H[hidx<3>(2, 2)] = d2;
+        H[hidx<3>(0, 1)] = e40 * q[1];
+        H[hidx<3>(0, 2)] = e40 * q[2];
+        H[hidx<3>(1, 2)] = e4 * q[1] * q[2];
+        G[0] = q[0] * d0;
+        G[1] = q[1] * d1;
+        G[2] = q[2] * d2;
     }
     __device__ __forceinline__ static double energy(const double* x, const SysPar& sp)
     {
