@@ -345,9 +345,24 @@ __device__ __forceinline__ void vector_step(const Slab<Sys>& sl, double* w, cons
     }
 }
 
+// 1 / (atol + rtol max(|x|, |xn|)), the weight of a component in the error norm.
+__device__ __forceinline__ double err_scale(const double x, const double xn, const double atol, const double rtol)
+{
+    return rcp_nr(fma(rtol, fmax(fabs(x), fabs(xn)), atol));
+}
+
+// The error of a trial from the weighted sums of squares over the D components
+// of h err5 and h err3: |h| E5 / sqrt(D (E5 + 0.01 E3)), 0 when both vanish.
+template <int D>
+__device__ __forceinline__ double err_of(const double E5, const double E3)
+{
+    if (E5 == 0.0 && E3 == 0.0) return 0.0;
+    return E5 * rsqrt_nr((double)D * fma(0.01, E3, E5));
+}
+
 // Error norm of a trial over the orbit components:
 //   scale_i = atol + rtol max(|x_i|, |xn_i|),  E5 = sum (err5_i / scale_i)^2,
-//   E3 likewise, err = |h| E5 / sqrt(D (E5 + 0.01 E3)) (0 when both vanish);
+//   E3 likewise, err = |h| E5 / sqrt(D (E5 + 0.01 E3));
 // e5 and e3 are h err5 and h err3, which absorbs the factor |h|.
 template <int D>
 __device__ __forceinline__ double err_norm(const double* x, const double* xn, const double* e5,
@@ -356,13 +371,12 @@ __device__ __forceinline__ double err_norm(const double* x, const double* xn, co
     double E5 = 0.0, E3 = 0.0;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-        const double rsc = 1.0 / (atol + rtol * fmax(fabs(x[i]), fabs(xn[i])));
+        const double rsc = err_scale(x[i], xn[i], atol, rtol);
         const double q5 = e5[i] * rsc, q3 = e3[i] * rsc;
         E5 = fma(q5, q5, E5);
         E3 = fma(q3, q3, E3);
     }
-    if (E5 == 0.0 && E3 == 0.0) return 0.0;
-    return E5 / sqrt((double)D * (E5 + 0.01 * E3));
+    return err_of<D>(E5, E3);
 }
 
 // SALI of two vectors (each normalised first): min(|u + v|, |u - v|).

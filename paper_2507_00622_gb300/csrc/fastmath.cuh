@@ -78,6 +78,37 @@ __device__ __forceinline__ double rsqrt_nr(double a)
     return rsqrt(a);
 }
 
+// 1/a for a > 0, relative error ~1e-13: the SFU's single-precision reciprocal and
+// one Newton step y + y (1 - a y) in FP64 (2 FP64 instructions); the division
+// outside the range in which the reciprocal is a normal float.
+__device__ __forceinline__ double rcp_nr(double a)
+{
+    const int hi = __double2hiint(a), lo = __double2loint(a);
+    if (in_f32_range(hi) && hi < ((1023 + 125) << 20)) {
+        float yf;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(f64_to_f32_trunc(hi, lo)));
+        const double y = f32_to_f64_bits(yf);
+        return fma(y, fma(-a, y, 1.0), y);
+    }
+    return 1.0 / a;
+}
+
+// a^(-1/8) for a > 0: single-precision exp2(-log2(a) / 8) (relative error ~1e-6)
+// and one Newton step y + y (1 - a y^8) / 8, whose error is 4.5 times the square
+// of the start's (~1e-11; a step size takes the factor, nothing else does); three
+// square roots and a division, ~60 FP64 instructions instead of 6, outside the
+// single-precision range and for a NaN.
+__device__ __forceinline__ double inv_root8(double a)
+{
+    const int hi = __double2hiint(a), lo = __double2loint(a);
+    if (in_f32_range(hi) && hi < ((1023 + 125) << 20)) {
+        const double y = f32_to_f64_bits(exp2f(-0.125f * log2f(f64_to_f32_trunc(hi, lo))));
+        const double y2 = y * y, y4 = y2 * y2;
+        return fma(0.125 * y, fma(-a * y4, y4, 1.0), y);
+    }
+    return 1.0 / sqrt(sqrt(sqrt(a)));
+}
+
 // --------------------------------------------------------------------------
 // Double-float arithmetic for the LD integrand and the renormalisation
 //

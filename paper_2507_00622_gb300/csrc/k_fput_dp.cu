@@ -8,8 +8,8 @@
 // running the 2N deviation vectors through the twelve stages side by side
 // would need 11 stage copies of the 2N x 2N matrix W (1.4 MB per orbit at
 // N = 64).  So a step runs in the two phases of fput_stages.cuh: the orbit
-// through its stages (one thread per component), then the columns of W one at
-// a time per warp segment, with their stage derivatives in registers.
+// through its stages (one thread per mass), then the columns of W one at
+// a time per warp segment, with their stage values in registers.
 //
 // W lives in shared memory column-major with a padded column stride 2N + 1, so
 // that both a warp reading down a column and the QR's thread-per-column sweeps
@@ -21,7 +21,7 @@
 // same in every thread), from which the orbit's first thread forms the error
 // and the step factor for all of its threads; the columns of W advance only
 // for accepted trials.  A block loops until all of its orbits are done.
-#include "fput_ens.cuh"
+#include "fput_stages.cuh"
 
 namespace chs {
 namespace {
@@ -32,9 +32,9 @@ struct FputDpCfg {
     static constexpr int G = D >= 32 ? 1 : 32 / D;  // orbits per block: one warp for N <= 16
     static constexpr int THREADS = G * D;             // 32, 64 or 128
     static constexpr int WS = D + 1;                   // padded column stride
-    // doubles per orbit: W, two stage-state buffers, 12 stage stiffness rows,
-    // two error-sum rows, control words
-    static constexpr int PER = D * WS + 2 * D + 12 * (N + 1) + 2 * D + 6 + (D == 128 ? 8 * D : 0);
+    // doubles per orbit: W, two stage-position buffers, 12 stage rows of bond
+    // stiffnesses and of their sums, warp partials, control words
+    static constexpr int PER = D * WS + 2 * N + 12 * (2 * N + 1) + 4 + 8 + (D == 128 ? 8 * D : 0);
     static constexpr size_t SMEM = (size_t)G * PER * sizeof(double);
     static_assert(THREADS % 32 == 0 && THREADS <= 128, "whole warps, N <= 64");
 };
@@ -44,12 +44,13 @@ template <int N>
 struct FputDpSlab {
     using Cfg = FputDpCfg<N>;
     static constexpr int W = 0;
-    static constexpr int XB = Cfg::D * Cfg::WS;     // [2][D]
-    static constexpr int CS = XB + 2 * Cfg::D;      // [12][N + 1]
-    static constexpr int ER = CS + 12 * (N + 1);    // [2][D] error sums
-    static constexpr int CTL = ER + 2 * Cfg::D;     // [0] red, [1] any, [2] step of phase 2, [3] advance,
-                                                    // [4] error, [5] err^(-1/8)
-    static constexpr int QP = CTL + 6;              // N = 64: the split QR's partial sums [2][4][D]
+    static constexpr int XB = Cfg::D * Cfg::WS;     // [2][N]
+    static constexpr int CS = XB + 2 * N;           // [12][N + 1]
+    static constexpr int DG = CS + 12 * (N + 1);    // [12][N]
+    static constexpr int ER = DG + 12 * N;          // [4] warp partials of orbit sums
+    static constexpr int CTL = ER + 4;              // [0] red, [1] any, [2] step of phase 2, [3] advance,
+                                                    // [4] error, [5] err^(-1/8), [6] 1 / step
+    static constexpr int QP = CTL + 8;              // N = 64: the split QR's partial sums [2][4][D]
     static_assert(QP + (Cfg::D == 128 ? 8 * Cfg::D : 0) == Cfg::PER, "slab layout");
 };
 
@@ -270,9 +271,10 @@ k_fput_lyap_dp(const StepArgs a, const SysPar sp, const int64_t n, const double*
     double* slab = smem + g * PER;
     double* red = slab + Sl::CTL;
 
-    const fs::Coef fc = fs::coef_of(sp);
+    const bool mass = l < N;  // thread l < N carries mass l
     int32_t st = valid ? (ic_status ? ic_status[o] : CHS_ORBIT_OK) : CHS_ORBIT_FORBIDDEN;
-    double xi = valid ? ics[(int64_t)l * n + o] : 0.0;
+    double q = (valid && mass) ? ics[(int64_t)l * n + o] : 0.0;
+    double p = (valid && mass) ? ics[(int64_t)(N + l) * n + o] : 0.0;
 
     // orbit-wide "any thread" (block-wide barriers; every thread takes part)
     auto orbit_any = [&](bool pred) {
@@ -284,23 +286,24 @@ k_fput_lyap_dp(const StepArgs a, const SysPar sp, const int64_t n, const double*
         __syncthreads();
         return r;
     };
-    if (orbit_any(!isfinite(xi)) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
-    if (st != CHS_ORBIT_OK) xi = 0.0;
+    if (orbit_any(!(isfinite(q) && isfinite(p))) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
+    if (st != CHS_ORBIT_OK) q = p = 0.0;
 
 #pragma unroll 4
     for (int i = 0; i < D; ++i) slab[Sl::W + l * WS + i] = (i == l) ? 1.0 : 0.0;
     double S = 0.0;
     __syncthreads();
 
-    const double h = a.dt;
+    const dp::StepH sh = dp::step_h(a.dt);
     int64_t until_qr = a.qr_every;
     int64_t until = a.sample_every > 0 ? a.sample_every : -1;
     const long long t_start = clock64();
     for (int64_t step = 1; step <= a.n_steps; ++step) {
-        double e5, e3;
-        xi = fs::orbit_stages<N, fs::TabDop853, false>(xi, h, l, slab + Sl::XB, slab + Sl::CS, fc, e5, e3);
+        fs::mass_stages<N, fs::TabDop853, false, Cfg::THREADS == 32>(q, p, sh, l, slab + Sl::XB, slab + Sl::CS,
+                                                                     slab + Sl::DG, sp, q, p, nullptr, mass);
         __syncthreads();  // every stage stiffness is written
-        fs::columns<N, fs::TabDop853, G, PER, WS, Sl::CS, false>(smem, D, [&](int, const double*) { return h; });
+        fs::columns<N, fs::TabDop853, G, PER, WS, Sl::CS, Sl::DG, false>(smem, D,
+                                                                         [&](int, const double*) { return sh; });
         __syncthreads();  // W complete; stage stiffnesses free
         if (--until_qr == 0 || step == a.n_steps) {
             until_qr = a.qr_every;
@@ -308,7 +311,7 @@ k_fput_lyap_dp(const StepArgs a, const SysPar sp, const int64_t n, const double*
         }
         if (--until == 0) {
             until = a.sample_every;
-            if (orbit_any(!(isfinite(xi) && isfinite(S))) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
+            if (orbit_any(!(isfinite(q) && isfinite(p) && isfinite(S))) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
             // block-uniform: the block's orbits stop together
             if (a.clock_budget > 0 && __syncthreads_or(budget_spent(a, t_start))) {
                 if (st == CHS_ORBIT_OK) st = CHS_ORBIT_STEP_BUDGET;
@@ -327,7 +330,7 @@ k_fput_lyap_dp(const StepArgs a, const SysPar sp, const int64_t n, const double*
 // N = 64 with 256 threads per orbit (one orbit per block and per SM, as in
 // k_fput_lyap_dp<64>): two warps per sub-partition instead of one, so that one
 // warp's shared-memory traffic and barriers overlap the other's FP64 work.  The
-// orbit's stages run on threads t < 128 exactly as in k_fput_lyap_dp (the others
+// orbit's stages run on threads t < 64 exactly as in k_fput_lyap_dp (the others
 // only meet the barriers); phase 2 spreads the 128 columns over 8 warps instead
 // of 4; the QR is qr_step_split_wide.  Every column, stage and dot product is
 // computed as in k_fput_lyap_dp<64>: identical results.
@@ -350,9 +353,10 @@ k_fput_lyap_dp_wide(const StepArgs a, const SysPar sp, const int64_t n, const do
     double* slab = smem;
     double* red = slab + Sl::CTL;
 
-    const fs::Coef fc = fs::coef_of(sp);
+    const bool mass = t < N;  // thread t < N carries mass t
     int32_t st = valid ? (ic_status ? ic_status[o] : CHS_ORBIT_OK) : CHS_ORBIT_FORBIDDEN;
-    double xi = (valid && lead) ? ics[(int64_t)l * n + o] : 0.0;
+    double q = (valid && mass) ? ics[(int64_t)t * n + o] : 0.0;
+    double p = (valid && mass) ? ics[(int64_t)(N + t) * n + o] : 0.0;
 
     auto orbit_any = [&](bool pred) {
         if (t == 0) red[1] = 0.0;
@@ -363,24 +367,24 @@ k_fput_lyap_dp_wide(const StepArgs a, const SysPar sp, const int64_t n, const do
         __syncthreads();
         return r;
     };
-    if (orbit_any(lead && !isfinite(xi)) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
-    if (st != CHS_ORBIT_OK) xi = 0.0;
+    if (orbit_any(!(isfinite(q) && isfinite(p))) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
+    if (st != CHS_ORBIT_OK) q = p = 0.0;
 
 #pragma unroll 4
     for (int i = 64 * half; i < 64 * half + 64; ++i) slab[Sl::W + l * WS + i] = (i == l) ? 1.0 : 0.0;
     double S = 0.0;
     __syncthreads();
 
-    const double h = a.dt;
+    const dp::StepH sh = dp::step_h(a.dt);
     int64_t until_qr = a.qr_every;
     int64_t until = a.sample_every > 0 ? a.sample_every : -1;
     const long long t_start = clock64();
     for (int64_t step = 1; step <= a.n_steps; ++step) {
-        double e5, e3;
-        xi = fs::orbit_stages<N, fs::TabDop853, false, true>(xi, h, l, slab + Sl::XB, slab + Sl::CS, fc, e5, e3,
-                                                             lead);
+        fs::mass_stages<N, fs::TabDop853, false, false>(q, p, sh, t, slab + Sl::XB, slab + Sl::CS, slab + Sl::DG, sp,
+                                                        q, p, nullptr, mass);
         __syncthreads();  // every stage stiffness is written
-        fs::columns<N, fs::TabDop853, 1, PER, WS, Sl::CS, false>(smem, D, [&](int, const double*) { return h; });
+        fs::columns<N, fs::TabDop853, 1, PER, WS, Sl::CS, Sl::DG, false>(smem, D,
+                                                                         [&](int, const double*) { return sh; });
         __syncthreads();  // W complete; stage stiffnesses free
         if (--until_qr == 0 || step == a.n_steps) {
             until_qr = a.qr_every;
@@ -388,7 +392,7 @@ k_fput_lyap_dp_wide(const StepArgs a, const SysPar sp, const int64_t n, const do
         }
         if (--until == 0) {
             until = a.sample_every;
-            if (orbit_any(lead && !(isfinite(xi) && isfinite(S))) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
+            if (orbit_any(lead && !(isfinite(q) && isfinite(p) && isfinite(S))) && st == CHS_ORBIT_OK) st = CHS_ORBIT_NONFINITE;
             // block-uniform: the orbit's threads stop together
             if (a.clock_budget > 0 && __syncthreads_or(budget_spent(a, t_start))) {
                 if (st == CHS_ORBIT_OK) st = CHS_ORBIT_STEP_BUDGET;
@@ -423,11 +427,12 @@ k_fput_lyap_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const i
     double* ctl = slab + Sl::CTL;
     double* er = slab + Sl::ER;
 
-    const fs::Coef fc = fs::coef_of(sp);
+    const bool mass = l < N;  // thread l < N carries mass l
     int32_t st = valid ? (ic_status ? ic_status[o] : CHS_ORBIT_OK) : CHS_ORBIT_FORBIDDEN;
-    double xi = valid ? ics[(int64_t)l * n + o] : 0.0;
+    double q = (valid && mass) ? ics[(int64_t)l * n + o] : 0.0;
+    double p = (valid && mass) ? ics[(int64_t)(N + l) * n + o] : 0.0;
     // a non-finite initial state is never accepted: it ends as STEP_FAIL
-    if (st != CHS_ORBIT_OK) xi = 0.0;
+    if (st != CHS_ORBIT_OK) q = p = 0.0;
 
 #pragma unroll 4
     for (int i = 0; i < D; ++i) slab[Sl::W + l * WS + i] = (i == l) ? 1.0 : 0.0;
@@ -469,33 +474,37 @@ k_fput_lyap_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const i
         }
         if (!__syncthreads_or(active)) break;
 
-        double e5 = 0.0, e3 = 0.0;
-        const double xn = fs::orbit_stages<N, fs::TabDop853, true>(xi, hh, l, slab + Sl::XB, slab + Sl::CS, fc, e5, e3);
-        // error norm over the orbit's components, summed in index order by
-        // every thread of the orbit
-        const double sc = ad.atol + ad.rtol * fmax(fabs(xi), fabs(xn));
-        const double q5 = e5 / sc, q3 = e3 / sc;
-        const double E5 = fe::orbit_sum<D>(q5 * q5, er, l);
-        const double E3 = fe::orbit_sum<D>(q3 * q3, er, l);
+        double nq, np, es[4];
+        const dp::StepH sh = dp::step_h(hh);
+        fs::mass_stages<N, fs::TabDop853, true, Cfg::THREADS == 32>(q, p, sh, l, slab + Sl::XB, slab + Sl::CS,
+                                                                    slab + Sl::DG, sp, nq, np, es, mass);
+        // error norm over the orbit's components
+        double s5 = 0.0, s3 = 0.0;
+        if (mass) fs::mass_error(q, p, nq, np, es, ad.atol, ad.rtol, s5, s3);
+        const double E5 = fs::orbit_sum<D>(s5, er, l);
+        const double E3 = fs::orbit_sum<D>(s3, er, l);
         if (l == 0) {
-            const double err =
-                (E5 == 0.0 && E3 == 0.0) ? 0.0 : fabs(hh) * E5 / sqrt((double)D * (E5 + 0.01 * E3));
-            ctl[2] = (active && err < 1.0) ? hh : 0.0;
+            const double err = dp::err_of<D>(E5, E3);
+            const bool ok = active && err < 1.0;
+            ctl[2] = ok ? hh : 0.0;
+            ctl[6] = ok ? sh.rh : 0.0;
             ctl[4] = err;
-            // err^(-1/8) as three square roots and a division
-            ctl[5] = (active && err > 0.0) ? 1.0 / sqrt(sqrt(sqrt(err))) : 0.0;
+            ctl[5] = (active && err > 0.0) ? inv_root8(err) : 0.0;
         }
         __syncthreads();  // stage stiffnesses, phase-2 steps and the error are in place
         const double err = ctl[4], r8 = ctl[5];
         const bool accept = active && err < 1.0;
 
-        fs::columns<N, fs::TabDop853, G, PER, WS, Sl::CS, true>(smem, D, [&](int, const double* sl) { return sl[Sl::CTL + 2]; });
+        fs::columns<N, fs::TabDop853, G, PER, WS, Sl::CS, Sl::DG, true>(smem, D, [&](int, const double* sl) {
+            return dp::StepH{sl[Sl::CTL + 2], 0.0, sl[Sl::CTL + 6]};
+        });
         if (active) {
             if (accept) {
                 double fac = (err == 0.0) ? 10.0 : fmin(10.0, 0.9 * r8);
                 if (rejected) fac = fmin(fac, 1.0);
                 hnext = hh * fac;
-                xi = xn;
+                q = nq;
+                p = np;
                 tt = tn;
                 ++done;
                 rejected = false;

@@ -4,8 +4,9 @@
 //
 // Every orbit has its own time and step size.  A trial advances the orbit
 // through the twelve stages (phase 1 of fput_stages.cuh); the error norm over
-// its 2N components is an orbit-wide sum that every thread of the orbit holds
-// bit for bit, so all of them take the same accept / reject decision.  The
+// its 2N components is an orbit-wide sum that every lane of the orbit holds
+// bit for bit, so all of them take the same accept / reject decision (lanes of
+// fput_ens.cuh).  The
 // deviation vectors advance (phase 2, renormalised with renorm) only for
 // accepted trials, and the checks of fput_ens.cuh follow each accepted step.
 // Controller: safety 0.9, growth at most 10 (not above 1 right after a
@@ -17,28 +18,23 @@ namespace chs {
 namespace {
 
 template <int N>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32)
 k_fput_ens_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const int K, const EnsPtrs e,
                  const AdaptPtrs ap)
 {
     using Tab = fs::TabDop853;
     using C = fe::Cfg<N, Tab>;
-    constexpr int D = C::D, G = C::G, PER = C::PER, WS = C::WS;
-    __shared__ double smem[G * PER];
-    const int g = threadIdx.x / D, l = threadIdx.x % D;
-    const int64_t n = e.n;
-    const int64_t o = (int64_t)blockIdx.x * G + g;
-    const bool valid = o < n;
-    double* slab = smem + g * PER;
-    double* red = slab + C::RED;
-    double* wg = static_cast<double*>(e.w);
-    const fs::Coef fc = fs::coef_of(sp);
+    constexpr int R = C::R;
+    extern __shared__ double smem[];
+    const fe::Lane<N, Tab> ln(smem);
+    const int64_t o = (int64_t)blockIdx.x * C::OPW + threadIdx.x / C::L;
+    const bool valid = o < e.n;
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
 
     int32_t st = valid ? e.status[o] : CHS_ORBIT_FORBIDDEN;
     const bool runs = st == CHS_ORBIT_OK;
-    double xi = valid ? e.x[(int64_t)l * n + o] : 0.0;
-    for (int j = 0; j < K; ++j) slab[C::W + j * WS + l] = valid ? wg[((int64_t)j * D + l) * n + o] : 0.0;
+    double q[R], p[R], nq[R], np[R];
+    ln.load(e, o, K, valid, q, p);
     const double h0 = runs ? e.h0[o] : 0.0;
     double dhm = runs ? e.dh_max[o] : 0.0;
     const int64_t exec0 = runs ? e.n_exec[o] : 0;
@@ -72,36 +68,25 @@ k_fput_ens_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const in
                 hh = tn - tt;
             }
         }
-        if (!__syncthreads_or(active)) break;
+        if (!__any_sync(fe::kFull, active)) break;
 
-        double e5 = 0.0, e3 = 0.0;
-        const double xn = fs::orbit_stages<N, Tab, true>(xi, hh, l, slab + C::XB, slab + C::CS, fc, e5, e3);
-        const double sc = ad.atol + ad.rtol * fmax(fabs(xi), fabs(xn));
-        const double q5 = e5 / sc, q3 = e3 / sc;
-        const double E5 = fe::orbit_sum<D>(q5 * q5, red, l);
-        const double E3 = fe::orbit_sum<D>(q3 * q3, red, l);
-        // the orbit's first thread forms the error and err^(-1/8) (three square
-        // roots and a division) for all of its threads, which read them back
-        // after the barrier: the other warps of a long chain skip that work
-        if (l == 0) {
-            const double err =
-                (E5 == 0.0 && E3 == 0.0) ? 0.0 : fabs(hh) * E5 / sqrt((double)D * (E5 + 0.01 * E3));
-            slab[C::CTL] = (active && err < 1.0) ? hh : 0.0;
-            slab[C::CTL + 1] = err;
-            slab[C::CTL + 2] = (active && err > 0.0) ? 1.0 / sqrt(sqrt(sqrt(err))) : 0.0;
-        }
-        __syncthreads();  // stage stiffnesses, phase-2 steps and the error in place
-        const double err = slab[C::CTL + 1], r8 = slab[C::CTL + 2];
+        const dp::StepH sh = dp::step_h(hh);
+        double s5, s3;
+        ln.template orbit_step<true>(q, p, sh, sp, nq, np, ad.atol, ad.rtol, s5, s3);
+        const double err = dp::err_of<C::D>(fe::lane_sum<C::L>(s5), fe::lane_sum<C::L>(s3));
+        const double r8 = (active && err > 0.0) ? inv_root8(err) : 0.0;
         const bool accept = active && err < 1.0;
-        fs::columns<N, Tab, G, PER, WS, C::CS, true>(smem, K, [](int, const double* sl) { return sl[C::CTL]; },
-                                               a.renorm);
-        __syncthreads();  // columns complete; stage buffers free
+        ln.vectors_step(K, accept ? sh : dp::StepH{0.0, 0.0, 0.0}, a.renorm);
         if (active) {
             if (accept) {
                 double fac = (err == 0.0) ? 10.0 : fmin(10.0, 0.9 * r8);
                 if (rejected) fac = fmin(fac, 1.0);
                 hnext = hh * fac;
-                xi = xn;
+#pragma unroll
+                for (int k = 0; k < R; ++k) {
+                    q[k] = nq[k];
+                    p[k] = np[k];
+                }
                 tt = tn;
                 el = err;
                 em = fmax(em, err);
@@ -116,17 +101,16 @@ k_fput_ens_adapt(const StepArgs a, const AdaptArgs ad, const SysPar sp, const in
             }
         }
         const bool check = accept && a.sample_every > 0 && (exec0 + done) % a.sample_every == 0;
-        const bool any_check = __syncthreads_or(check);
-        st = fe::post_step<N, Tab>(a, sp, K, slab, l, xi, accept, check, any_check, h0, dhm, st);
-        if (any_check && a.clock_budget > 0) {  // block-uniform: the block's orbits stop together
-            const bool over = __syncthreads_or(budget_spent(a, t_start)) != 0;
+        const bool any_check = __any_sync(fe::kFull, check);
+        st = ln.post_step(a, sp, K, q, p, accept, check, any_check, h0, dhm, st);
+        if (any_check && a.clock_budget > 0) {  // warp-uniform: the warp's orbits stop together
+            const bool over = __any_sync(fe::kFull, budget_spent(a, t_start)) != 0;
             if (over && check && st == CHS_ORBIT_OK) st = CHS_ORBIT_STEP_BUDGET;
         }
     }
     if (runs) {
-        e.x[(int64_t)l * n + o] = xi;
-        for (int j = 0; j < K; ++j) wg[((int64_t)j * D + l) * n + o] = slab[C::W + j * WS + l];
-        if (l == 0) {
+        ln.store(e, o, K, q, p);
+        if (ln.first) {
             e.dh_max[o] = dhm;
             e.n_exec[o] = exec0 + done;
             e.status[o] = st;
@@ -144,7 +128,7 @@ cudaError_t adapt_n(const SysPar& sp, int k, const StepArgs& a, const AdaptArgs&
                     const AdaptPtrs& ap, cudaStream_t st)
 {
     using C = fe::Cfg<N, fs::TabDop853>;
-    k_fput_ens_adapt<N><<<blocks_for(e.n, C::G), C::THREADS, 0, st>>>(a, ad, sp, k, e, ap);
+    k_fput_ens_adapt<N><<<blocks_for(e.n, C::OPW), 32, C::smem(k), st>>>(a, ad, sp, k, e, ap);
     return cudaGetLastError();
 }
 
