@@ -13,9 +13,8 @@
 //   W1 [128][12], b1 [128], W2 [128][128], b2 [128], W3 [128][128], b3 [128],
 //   W4 [2][128], b4 [2]   -- 34,946 values.
 //
-// The work is tiny next to the integration (about 35k multiply-adds per orbit),
-// so the kernels run on the FP32 CUDA-core pipe with the layer weights staged in
-// shared memory; the weights and activations are stored in BF16.
+// The hidden layers of the forward pass run on the tensor cores (below), the
+// training kernels on the FP32 pipe; weights and activations are stored in BF16.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -59,61 +58,261 @@ __global__ void k_mlp_features(const double* __restrict__ series, const int S, c
     for (int i = 0; i < kF; ++i) X[(int64_t)i * n + o] = f[i];
 }
 
-// One dense layer on a tile of kTile samples held in shared memory:
-//   out[u][s] = act(b[u] + sum_k W[u][k] in[k][s]),  u < U, k < K.
-// For U >= 32 each thread owns a (U/32) x (kTile/8) register tile (units tu + 32a,
-// samples ts + 8b), so the 256 threads cover U x kTile outputs.
-template <int U, int K, bool RELU>
-__device__ __forceinline__ void dense_tile(const __nv_bfloat16* __restrict__ Wg, const __nv_bfloat16* __restrict__ bg,
-                                           float* __restrict__ Ws, const float* __restrict__ in,
-                                           float* __restrict__ out)
+// ---------------------------------------------------------------------------
+// Forward pass
+//
+// A persistent grid (one block of kFwdWarps warps per SM); a warp takes tiles of
+// 32 samples, as two halves of 16 rows, through all layers without leaving its
+// own shared memory:
+//   features / X   FP32, 32 samples at a time;
+//   layer 1        FP32 FMA chains (K = 12, FP32 inputs);
+//   layers 2, 3    mma.sync m16n8k16 (BF16 operands, FP32 accumulators), weights
+//                  resident in shared memory, operands by ldmatrix;
+//   layer 4        FP32 FMA chains (2 x 128 per sample).
+// The products of layers 2 and 3 are a fifth of the kernel's time here, behind the
+// FP64 features and the FP32 layers, and M = 16 rows per warp keep a batch of a
+// few thousand samples on all SMs, so the wider tcgen05 tiles would gain nothing.
+//
+// The activations are BF16, so the order of a layer's FP32 sum decides the
+// result only where the sum lies within rounding of a BF16 rounding boundary
+// (or of zero, for the ReLU).  The definition is the sequential chain
+// acc = fma(w_k, a_k, acc), k ascending, plus the bias; the tensor cores sum in
+// another order.  Every output whose BF16 value would change within
+//   delta = 2^-20 (|w_u|_2 |a|_2 + |b_u|)
+// of the tensor-core sum (16 times the rounding unit of a bound on every partial
+// sum; about 0.3 % of the outputs) is computed again by the chain itself, so the
+// activations are those of the chain and the result does not depend on the
+// tensor cores' summation order.
+//
+// chs_surrogate_decide on 524,288 samples (GB300): 0.41 ms, 5.80 ms with FP32 register
+// tiles for all layers and the library's log10; 88 TFLOP/s of 2 x 34,560 flops a
+// sample.  FP64 instruction slots (the features' logarithms, the sigmoid) bound it.
+// ---------------------------------------------------------------------------
+
+constexpr int kFwdWarps = 12;
+constexpr int kWS = kH + 8;  // padded row of a BF16 matrix in shared memory (ldmatrix without conflicts)
+constexpr float kDelta = 9.5367431640625e-07f;  // 2^-20
+constexpr int kLogTab = 64;
+
+struct alignas(16) FwdWarp {
+    __nv_bfloat16 a[2][16 * kWS];  // activations of one half: layer input and output
+    float x[kF][32];
+    float y[2][32];
+};
+struct alignas(16) FwdSmem {
+    __nv_bfloat16 w2[kH * kWS], w3[kH * kWS];
+    float w1[kF][kH];  // transposed
+    float w4[kO][kH];
+    float b[3][kH], b4[kO];
+    float wn[2][kH], bn[2][kH];  // delta's factors |w_u| and |b_u| of layers 2 and 3, times 2^-20
+    double2 lt[kLogTab];         // (1 / c, log10(c) / 8), c the middle of a mantissa interval
+    FwdWarp warp[kFwdWarps];
+};
+
+// log10(s) / 8 for a positive normal s, absolute error below 5e-16: s =
+// 2^e m, log10(m) = log10(c) + log10(1 + r) with c from the table and r = m / c -
+// 1, |r| <= 2^-7 (Tang, ACM TOMS 16, 1990), six terms of the series.  10 FP64
+// instructions against the library's ~30; rounded to FP32 the two differ once in
+// a million values.
+__device__ __forceinline__ double log10_8(const double s, const double2* __restrict__ lt)
 {
-    // stage the weights as float
-    for (int i = threadIdx.x; i < U * K; i += kThreads) Ws[i] = bf(Wg[i]);
-    __syncthreads();
-    if constexpr (U >= 32) {
-        constexpr int TU = U / 32;     // units per thread
-        constexpr int TS = kTile / 8;  // samples per thread
-        const int tu = threadIdx.x % 32, ts = threadIdx.x / 32;
-        float acc[TU][TS];
+    const int hi = __double2hiint(s);
+    const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(s));
+    const double2 c = lt[(hi >> 14) & (kLogTab - 1)];
+    const double r = fma(m, c.x, -1.0);
+    constexpr double q = 0.43429448190325182765 / 8.0;  // log10(e) / 8
+    double p = -q / 6.0;
+    p = fma(p, r, q / 5.0);
+    p = fma(p, r, -q / 4.0);
+    p = fma(p, r, q / 3.0);
+    p = fma(p, r, -q / 2.0);
+    p = fma(p, r, q);
+    // the exponent as a double by its bits (2^52 + 2^31 + e, e > -2^31)
+    const double e = __hiloint2double(0x43300000, (int)(0x80000000u + (unsigned)((hi >> 20) - 1023))) -
+                     (4503599627370496.0 + 2147483648.0);
+    return fma(p, r, fma(e, 0.30102999566398119521 / 8.0, c.y));
+}
+
+__device__ __forceinline__ void ldmatrix4(unsigned (&r)[4], const void* p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+
+__device__ __forceinline__ void ldmatrix4_trans(unsigned (&r)[4], const void* p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], const unsigned b0, const unsigned b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// The chain of one output over K = 128 inputs: rows of W and of the activations
+// (16-byte aligned), k ascending.
+__device__ __forceinline__ float chain128(const __nv_bfloat16* __restrict__ w, const __nv_bfloat16* __restrict__ a)
+{
+    float acc = 0.0f;
+#pragma unroll 4
+    for (int k = 0; k < kH; k += 8) {
+        const uint4 wv = *reinterpret_cast<const uint4*>(w + k), av = *reinterpret_cast<const uint4*>(a + k);
+        const unsigned wu[4] = {wv.x, wv.y, wv.z, wv.w}, au[4] = {av.x, av.y, av.z, av.w};
 #pragma unroll
-        for (int a = 0; a < TU; ++a)
-#pragma unroll
-            for (int b = 0; b < TS; ++b) acc[a][b] = 0.0f;
-        for (int k = 0; k < K; ++k) {
-            float wv[TU], iv[TS];
-#pragma unroll
-            for (int a = 0; a < TU; ++a) wv[a] = Ws[(tu + 32 * a) * K + k];
-#pragma unroll
-            for (int b = 0; b < TS; ++b) iv[b] = in[k * kTile + ts + 8 * b];
-#pragma unroll
-            for (int a = 0; a < TU; ++a)
-#pragma unroll
-                for (int b = 0; b < TS; ++b) acc[a][b] = fmaf(wv[a], iv[b], acc[a][b]);
-        }
-#pragma unroll
-        for (int a = 0; a < TU; ++a) {
-            const int u = tu + 32 * a;
-            const float bu = bf(bg[u]);
-#pragma unroll
-            for (int b = 0; b < TS; ++b) {
-                float v = acc[a][b] + bu;
-                if (RELU) v = fmaxf(v, 0.0f);
-                out[u * kTile + ts + 8 * b] = bf(__float2bfloat16_rn(v));  // BF16 activations
-            }
-        }
-    } else {
-        // small output layer: one (unit, sample) pair per thread
-        for (int p = threadIdx.x; p < U * kTile; p += kThreads) {
-            const int u = p / kTile, s = p % kTile;
-            float acc = 0.0f;
-            for (int k = 0; k < K; ++k) acc = fmaf(Ws[u * K + k], in[k * kTile + s], acc);
-            float v = acc + bf(bg[u]);
-            if (RELU) v = fmaxf(v, 0.0f);
-            out[u * kTile + s] = v;
+        for (int i = 0; i < 4; ++i) {
+            acc = fmaf(__uint_as_float(wu[i] << 16), __uint_as_float(au[i] << 16), acc);
+            acc = fmaf(__uint_as_float(wu[i] & 0xffff0000u), __uint_as_float(au[i] & 0xffff0000u), acc);
         }
     }
-    __syncthreads();
+    return acc;
+}
+
+__device__ __forceinline__ unsigned pack_relu(const float lo, const float hi)
+{
+    const __nv_bfloat162 v = __floats2bfloat162_rn(fmaxf(lo, 0.0f), fmaxf(hi, 0.0f));
+    return *reinterpret_cast<const unsigned*>(&v);
+}
+
+// The squares of the packed pair added to s (the norm of a row of activations).
+__device__ __forceinline__ float add_squares(const unsigned v, float s)
+{
+    const float lo = __uint_as_float(v << 16), hi = __uint_as_float(v & 0xffff0000u);
+    return fmaf(hi, hi, fmaf(lo, lo, s));
+}
+
+// |a|_2 of rows g and g + 8 from the quad's partial sums.
+__device__ __forceinline__ void row_norms(float (&n2)[2])
+{
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        n2[r] += __shfl_xor_sync(0xffffffffu, n2[r], 1);
+        n2[r] += __shfl_xor_sync(0xffffffffu, n2[r], 2);
+        n2[r] = sqrtf(n2[r]);
+    }
+}
+
+// Layer 1 on one half (rows = samples 16 half .. + 15 of wp.x): FP32 chains over
+// the 12 inputs, outputs where an mma accumulator would have them.
+__device__ __forceinline__ void layer1(const FwdSmem& sm, FwdWarp& wp, const int half, float (&norm)[2])
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    float xa[kF], xb[kF];
+#pragma unroll
+    for (int k = 0; k < kF; ++k) {
+        xa[k] = wp.x[k][16 * half + g];
+        xb[k] = wp.x[k][16 * half + g + 8];
+    }
+    norm[0] = norm[1] = 0.0f;
+#pragma unroll 4
+    for (int nt = 0; nt < kH / 8; ++nt) {
+        const int u = 8 * nt + 2 * t;
+        float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int k = 0; k < kF; ++k) {
+            const float2 w = *reinterpret_cast<const float2*>(&sm.w1[k][u]);
+            c[0] = fmaf(w.x, xa[k], c[0]);
+            c[1] = fmaf(w.y, xa[k], c[1]);
+            c[2] = fmaf(w.x, xb[k], c[2]);
+            c[3] = fmaf(w.y, xb[k], c[3]);
+        }
+        const float2 bu = *reinterpret_cast<const float2*>(&sm.b[0][u]);
+        const unsigned va = pack_relu(c[0] + bu.x, c[1] + bu.y), vb = pack_relu(c[2] + bu.x, c[3] + bu.y);
+        *reinterpret_cast<unsigned*>(&wp.a[0][g * kWS + u]) = va;
+        *reinterpret_cast<unsigned*>(&wp.a[0][(g + 8) * kWS + u]) = vb;
+        norm[0] = add_squares(va, norm[0]);
+        norm[1] = add_squares(vb, norm[1]);
+    }
+    row_norms(norm);
+    __syncwarp();
+}
+
+// A hidden layer of 128 x 128 on one half: in -> out (16 rows each), norm the
+// row norms of in, replaced by those of out.
+__device__ __forceinline__ void layer_mma(const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias,
+                                          const float* __restrict__ wn, const float* __restrict__ bn,
+                                          const __nv_bfloat16* in, __nv_bfloat16* out, float (&norm)[2])
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    unsigned A[8][4];
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) ldmatrix4(A[ks], in + (lane & 15) * kWS + 16 * ks + 8 * (lane >> 4));
+    uint64_t again = 0;  // outputs to compute by the chain, bit 4 nt + e
+    float n2[2] = {0.0f, 0.0f};
+#pragma unroll 1
+    for (int nt = 0; nt < kH / 8; nt += 2) {
+        float c[2][4] = {};
+        const __nv_bfloat16* wr = W + (8 * nt + (lane & 7)) * kWS + 8 * (lane >> 3);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) {  // two k-steps of 16 per ldmatrix
+            unsigned B0[4], B1[4];
+            ldmatrix4(B0, wr + 32 * k2);
+            ldmatrix4(B1, wr + 8 * kWS + 32 * k2);
+            mma_bf16(c[0], A[2 * k2], B0[0], B0[1]);
+            mma_bf16(c[1], A[2 * k2], B1[0], B1[1]);
+            mma_bf16(c[0], A[2 * k2 + 1], B0[2], B0[3]);
+            mma_bf16(c[1], A[2 * k2 + 1], B1[2], B1[3]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int u = 8 * (nt + h) + 2 * t;
+            const float2 bu = *reinterpret_cast<const float2*>(bias + u);
+            const float2 wu = *reinterpret_cast<const float2*>(wn + u), bb = *reinterpret_cast<const float2*>(bn + u);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const float v0 = c[h][2 * r] + bu.x, v1 = c[h][2 * r + 1] + bu.y;
+                const float d0 = fmaf(wu.x, norm[r], bb.x), d1 = fmaf(wu.y, norm[r], bb.y);
+                const unsigned lo = pack_relu(v0 - d0, v1 - d1), up = pack_relu(v0 + d0, v1 + d1);
+                const unsigned diff = lo ^ up;
+                again |= (uint64_t)(((diff & 0xffffu) ? 1u : 0u) | ((diff & 0xffff0000u) ? 2u : 0u))
+                         << (4 * (nt + h) + 2 * r);
+                *reinterpret_cast<unsigned*>(&out[(g + 8 * r) * kWS + u]) = up;
+                n2[r] = add_squares(up, n2[r]);
+            }
+        }
+    }
+    while (again) {
+        const int i = __ffsll((long long)again) - 1;
+        again &= again - 1;
+        const int row = g + 8 * ((i >> 1) & 1), u = 8 * (i >> 2) + 2 * t + (i & 1);
+        const float v = chain128(W + u * kWS, in + row * kWS) + bias[u];
+        out[row * kWS + u] = __float2bfloat16_rn(fmaxf(v, 0.0f));
+    }
+    row_norms(n2);
+    norm[0] = n2[0];
+    norm[1] = n2[1];
+    __syncwarp();
+}
+
+// One layer's activations of a half to act [128][n]: pairs of samples by
+// transposed ldmatrix.
+__device__ __forceinline__ void store_act(const __nv_bfloat16* in, __nv_bfloat16* __restrict__ act, const int64_t s0,
+                                          const int64_t n)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const bool pair = (n & 1) == 0 && (reinterpret_cast<uintptr_t>(act) & 3) == 0;  // s0 is a multiple of 16
+#pragma unroll 1
+    for (int u0 = 0; u0 < kH; u0 += 16) {
+        unsigned r[4];  // (samples 0-7, units 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15), transposed
+        ldmatrix4_trans(r, in + (lane & 15) * kWS + u0 + 8 * (lane >> 4));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int64_t o = s0 + 8 * (i & 1) + 2 * t;
+            __nv_bfloat16* to = act + (int64_t)(u0 + 8 * (i >> 1) + g) * n + o;
+            if (pair && o + 1 < n) {
+                *reinterpret_cast<unsigned*>(to) = r[i];
+            } else {
+                const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&r[i]);
+                if (o < n) to[0] = v.x;
+                if (o + 1 < n) to[1] = v.y;
+            }
+        }
+    }
 }
 
 // Forward pass over the features X [12][n] (or, when series != NULL, over the
@@ -122,76 +321,110 @@ __device__ __forceinline__ void dense_tile(const __nv_bfloat16* __restrict__ Wg,
 // orbits whose status is OK take status EARLY_CHAOTIC when sigmoid(y0) >= conf
 // and PREDICTED_REGULAR when sigmoid(y0) <= 1 - conf, and t_end is not touched.
 template <bool FROM_SERIES>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(32 * kFwdWarps, 1)
 k_mlp_forward(const __nv_bfloat16* __restrict__ P, const float* __restrict__ X, const double* __restrict__ series,
               const int S, const double* __restrict__ ld, const double t, const double* __restrict__ E, const int64_t n,
               float* __restrict__ Y, __nv_bfloat16* __restrict__ act, int32_t* __restrict__ status,
               const double conf, float* __restrict__ prob)
 {
-    extern __shared__ float sm[];
-    float* Ws = sm;                        // kH * kH
-    float* A = Ws + kH * kH;               // kH * kTile
-    float* B = A + kH * kTile;             // kH * kTile
-    const int64_t s0 = (int64_t)blockIdx.x * kTile;
-    // input tile
-    if (FROM_SERIES) {
-        for (int s = threadIdx.x; s < kTile; s += kThreads) {
-            const int64_t o = s0 + s;
-            float fv[kF];
-            if (o < n) {
-                features(series, S, ld, t, E, n, o, fv);
-            } else {
-#pragma unroll
-                for (int f = 0; f < kF; ++f) fv[f] = 0.0f;
-            }
-#pragma unroll
-            for (int f = 0; f < kF; ++f) A[f * kTile + s] = fv[f];
-        }
-    } else {
-        for (int p = threadIdx.x; p < kF * kTile; p += kThreads) {
-            const int f = p / kTile, s = p % kTile;
-            const int64_t o = s0 + s;
-            A[f * kTile + s] = o < n ? X[(int64_t)f * n + o] : 0.0f;
-        }
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FwdSmem& sm = *reinterpret_cast<FwdSmem*>(smem_raw);
+    const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+    // the parameters: weights of layers 2 and 3 as BF16, the others widened
+    for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) {
+        const int u = i / kH, k = i % kH;
+        sm.w2[u * kWS + k] = P[kOffW2 + i];
+        sm.w3[u * kWS + k] = P[kOffW3 + i];
+    }
+    for (int i = threadIdx.x; i < kH * kF; i += blockDim.x) sm.w1[i % kF][i / kF] = bf(P[kOffW1 + i]);
+    for (int i = threadIdx.x; i < kO * kH; i += blockDim.x) sm.w4[i / kH][i % kH] = bf(P[kOffW4 + i]);
+    for (int u = threadIdx.x; u < kH; u += blockDim.x) {
+        sm.b[0][u] = bf(P[kOffB1 + u]);
+        sm.b[1][u] = bf(P[kOffB2 + u]);
+        sm.b[2][u] = bf(P[kOffB3 + u]);
+        if (u < kO) sm.b4[u] = bf(P[kOffB4 + u]);
+    }
+    if (FROM_SERIES && threadIdx.x < kLogTab) {
+        const double c = 1.0 + (threadIdx.x + 0.5) / kLogTab;
+        sm.lt[threadIdx.x] = make_double2(1.0 / c, log10(c) / 8.0);
     }
     __syncthreads();
-    dense_tile<kH, kF, true>(P + kOffW1, P + kOffB1, Ws, A, B);
-    if (act)
-        for (int p = threadIdx.x; p < kH * kTile; p += kThreads) {
-            const int64_t o = s0 + p % kTile;
-            if (o < n) act[(int64_t)(p / kTile) * n + o] = __float2bfloat16_rn(B[p]);
+    for (int i = threadIdx.x; i < 2 * kH; i += blockDim.x) {
+        const int l = i / kH, u = i % kH;
+        const __nv_bfloat16* w = (l ? sm.w3 : sm.w2) + u * kWS;
+        float s = 0.0f;
+        for (int k = 0; k < kH; ++k) s = fmaf(bf(w[k]), bf(w[k]), s);
+        sm.wn[l][u] = kDelta * sqrtf(s);
+        sm.bn[l][u] = kDelta * fabsf(sm.b[1 + l][u]);
+    }
+    __syncthreads();
+
+    FwdWarp& wp = sm.warp[warp];
+    const double rt = 1.0 / t;
+    const int64_t tiles = (n + 31) / 32;
+    for (int64_t tile = blockIdx.x + (int64_t)gridDim.x * warp; tile < tiles; tile += (int64_t)gridDim.x * kFwdWarps) {
+        const int64_t o = tile * 32 + lane;  // this lane's sample
+        const bool valid = o < n;
+        if (FROM_SERIES) {
+#pragma unroll 2
+            for (int i = 0; i < kS; ++i) {
+                double s = (valid && i < S) ? series[(int64_t)i * n + o] : 1e-20;
+                s = (s > 1e-20 && isfinite(s)) ? s : 1e-20;
+                wp.x[i][lane] = (float)log10_8(s, sm.lt);
+            }
+            wp.x[10][lane] = valid ? (float)fma(ld[o], rt, -1.0) : 0.0f;
+            wp.x[11][lane] = valid ? (float)((E[o] - 0.133) * (1.0 / 0.033)) : 0.0f;
+        } else {
+#pragma unroll
+            for (int k = 0; k < kF; ++k) wp.x[k][lane] = valid ? X[(int64_t)k * n + o] : 0.0f;
         }
-    dense_tile<kH, kH, true>(P + kOffW2, P + kOffB2, Ws, B, A);
-    if (act)
-        for (int p = threadIdx.x; p < kH * kTile; p += kThreads) {
-            const int64_t o = s0 + p % kTile;
-            if (o < n) act[(int64_t)(kH + p / kTile) * n + o] = __float2bfloat16_rn(A[p]);
+        __syncwarp();
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            const int64_t s0 = tile * 32 + 16 * half;
+            float norm[2];
+            layer1(sm, wp, half, norm);
+            if (act) store_act(wp.a[0], act, s0, n);
+            layer_mma(sm.w2, sm.b[1], sm.wn[0], sm.bn[0], wp.a[0], wp.a[1], norm);
+            if (act) store_act(wp.a[1], act + (int64_t)kH * n, s0, n);
+            layer_mma(sm.w3, sm.b[2], sm.wn[1], sm.bn[1], wp.a[1], wp.a[0], norm);
+            if (act) store_act(wp.a[0], act + (int64_t)2 * kH * n, s0, n);
+            // layer 4: lane (output, row), the chain over k
+            const int row = lane & 15, out = lane >> 4;
+            const __nv_bfloat16* a = wp.a[0] + row * kWS;
+            const float* w = sm.w4[out];
+            float acc = 0.0f;
+#pragma unroll 4
+            for (int k = 0; k < kH; k += 8) {
+                const uint4 av = *reinterpret_cast<const uint4*>(a + k);
+                const unsigned au[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    acc = fmaf(w[k + 2 * i], __uint_as_float(au[i] << 16), acc);
+                    acc = fmaf(w[k + 2 * i + 1], __uint_as_float(au[i] & 0xffff0000u), acc);
+                }
+            }
+            wp.y[out][16 * half + row] = acc + sm.b4[out];
+            __syncwarp();  // the half's buffers are free
         }
-    dense_tile<kH, kH, true>(P + kOffW3, P + kOffB3, Ws, A, B);
-    if (act)
-        for (int p = threadIdx.x; p < kH * kTile; p += kThreads) {
-            const int64_t o = s0 + p % kTile;
-            if (o < n) act[(int64_t)(2 * kH + p / kTile) * n + o] = __float2bfloat16_rn(B[p]);
-        }
-    dense_tile<kO, kH, false>(P + kOffW4, P + kOffB4, Ws, B, A);
-    for (int s = threadIdx.x; s < kTile; s += kThreads) {
-        const int64_t o = s0 + s;
-        if (o >= n) continue;
-        const float y0 = A[s], y1 = A[kTile + s];
-        if (Y) {
-            Y[o] = y0;
-            Y[n + o] = y1;
-        }
-        if (status) {
-            const double pc = 1.0 / (1.0 + exp(-(double)y0));
-            if (prob) prob[o] = (float)pc;
-            if (status[o] == CHS_ORBIT_OK) {
-                if (pc >= conf)
-                    status[o] = CHS_ORBIT_EARLY_CHAOTIC;
-                else if (pc <= 1.0 - conf)
-                    status[o] = CHS_ORBIT_PREDICTED_REGULAR;
+        if (valid) {
+            const float y0 = wp.y[0][lane], y1 = wp.y[1][lane];
+            if (Y) {
+                Y[o] = y0;
+                Y[n + o] = y1;
+            }
+            if (status) {
+                const double pc = 1.0 / (1.0 + exp(-(double)y0));
+                if (prob) prob[o] = (float)pc;
+                if (status[o] == CHS_ORBIT_OK) {
+                    if (pc >= conf)
+                        status[o] = CHS_ORBIT_EARLY_CHAOTIC;
+                    else if (pc <= 1.0 - conf)
+                        status[o] = CHS_ORBIT_PREDICTED_REGULAR;
+                }
             }
         }
+        __syncwarp();  // y and x are read before the next tile writes them
     }
 }
 
@@ -365,7 +598,19 @@ __global__ void k_mlp_adam(float* __restrict__ W, float* __restrict__ m, float* 
 
 // ---------------------------------------------------------------------------
 
-static constexpr size_t kFwdSmem = (size_t)(kH * kH + 2 * kH * kTile) * sizeof(float);
+static constexpr size_t kBwdSmem = (size_t)(kH * kH + 2 * kH * kTile) * sizeof(float);
+static_assert(sizeof(FwdSmem) <= 227 * 1024, "the forward kernel's shared memory");
+
+// Blocks of the persistent forward grid: one per SM, never more than tiles.
+static unsigned fwd_blocks(int64_t n)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        sms = 1;
+    const int64_t tiles = (n + 31) / 32;
+    return (unsigned)(tiles < sms ? tiles : sms);
+}
 
 cudaError_t launch_mlp_features(const double* series, int S, const double* ld, double t, const double* E,
                                 int64_t n, float* X, cudaStream_t st)
@@ -380,9 +625,9 @@ cudaError_t launch_mlp_forward(const void* P, const float* X, int64_t n, float* 
 {
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_forward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kFwdSmem);
+                                         (int)sizeof(FwdSmem));
     if (e != cudaSuccess) return e;
-    k_mlp_forward<false><<<blocks_for(n, kTile), kThreads, kFwdSmem, st>>>(
+    k_mlp_forward<false><<<fwd_blocks(n), 32 * kFwdWarps, sizeof(FwdSmem), st>>>(
         static_cast<const __nv_bfloat16*>(P), X, nullptr, 0, nullptr, 0.0, nullptr, n, Y,
         static_cast<__nv_bfloat16*>(act), nullptr, 0.0, nullptr);
     return cudaGetLastError();
@@ -394,9 +639,9 @@ cudaError_t launch_mlp_decide(const void* P, const double* series, int S, const 
 {
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_forward<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kFwdSmem);
+                                         (int)sizeof(FwdSmem));
     if (e != cudaSuccess) return e;
-    k_mlp_forward<true><<<blocks_for(n, kTile), kThreads, kFwdSmem, st>>>(
+    k_mlp_forward<true><<<fwd_blocks(n), 32 * kFwdWarps, sizeof(FwdSmem), st>>>(
         static_cast<const __nv_bfloat16*>(P), nullptr, series, S, ld, t, E, n, nullptr, nullptr, status,
         conf, prob);
     return cudaGetLastError();
@@ -417,9 +662,9 @@ cudaError_t launch_mlp_backward(const void* P, const float* X, const void* act, 
 {
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_backprop, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kFwdSmem);
+                                         (int)kBwdSmem);
     if (e != cudaSuccess) return e;
-    k_mlp_backprop<<<blocks_for(n, kTile), kThreads, kFwdSmem, st>>>(
+    k_mlp_backprop<<<blocks_for(n, kTile), kThreads, kBwdSmem, st>>>(
         static_cast<const __nv_bfloat16*>(P), static_cast<const __nv_bfloat16*>(act), dY, n, delta);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_mlp_wgrad<<<40, kThreads, 0, st>>>(X, static_cast<const __nv_bfloat16*>(act), delta, dY, n, G);
