@@ -136,6 +136,19 @@ chs_status check_ensemble(const chs_ensemble* e, const chs_params* p)
     return ok();
 }
 
+// High word of a bound on |q_i| below sqrt(escape_r2 / 3): while every |q_i| of an
+// orbit with at most three degrees of freedom lies below it, sum_i q_i^2 <
+// escape_r2.  Truncating to the high word lowers it; 0x7fffffff, which no |q_i|
+// reaches, with the test off.
+int escape_hi(const double escape_r2)
+{
+    if (!(escape_r2 > 0.0)) return 0x7fffffff;
+    const double bound = sqrt(escape_r2 / 3.0) * (1.0 - 1e-12);
+    int64_t bits;
+    memcpy(&bits, &bound, sizeof bits);
+    return (int)(bits >> 32);
+}
+
 chs::StepArgs step_args(const chs_params* p)
 {
     chs::StepArgs a;
@@ -148,6 +161,7 @@ chs::StepArgs step_args(const chs_params* p)
     a.ld_sqrt = p->ld_p == 0.5 ? 1 : 0;
     a.ld_p = p->ld_p;
     a.escape_r2 = p->escape_r2;
+    a.escape_hi = escape_hi(p->escape_r2);
     a.dh_limit = p->dh_limit;
     a.early_exit = p->early_exit;
     a.sali_threshold = p->sali_threshold;

@@ -62,6 +62,7 @@ struct StepArgs {
     int32_t ld_sqrt;       // 1: LD exponent is exactly 1/2 (sqrt path)
     double ld_p;
     double escape_r2;      // 0: off
+    int escape_hi;         // high word of a bound below sqrt(escape_r2 / 3) (0x7fffffff with the test off)
     double dh_limit;       // 0: off
     int32_t early_exit;    // freeze as EARLY_CHAOTIC once SALI < sali_threshold
     double sali_threshold;

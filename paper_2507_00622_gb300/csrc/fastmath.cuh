@@ -145,6 +145,14 @@ __device__ __forceinline__ FF ff_split(double a)
     return FF{hi, lo};
 }
 
+// ff_split for either sign.
+__device__ __forceinline__ FF ff_split_signed(double a)
+{
+    const FF m = ff_split(fabs(a));
+    const int sgn = __double2hiint(a) & (int)0x80000000;
+    return FF{__int_as_float(__float_as_int(m.hi) ^ sgn), __int_as_float(__float_as_int(m.lo) ^ sgn)};
+}
+
 // Exact widening of a finite float of either sign to double (integer pipe);
 // zero and subnormal floats give 0.
 __device__ __forceinline__ double f32_to_f64_signed(float f)
@@ -195,10 +203,22 @@ __device__ __forceinline__ FF ff_sum_sqrt_abs(const double* f)
     return acc;
 }
 
-// 1 / sqrt(a) for a > 0 in the FP32 exponent range, relative error ~2^-43, with
-// one FP64 addition: y ~ 1/sqrt(hi) from the SFU, e = 1 - a y^2 in double-float
-// (hi y = p + p_lo exactly by an FMA), result y + y e / 2.  Falls back to the
-// library rsqrt outside that range.
+// y + c as a double for normal floats y in [2^-75, 2^126] and |c| <= 2^-22 |y|, on the
+// integer pipe: c in units of the last place of the double y, added to its bits
+// (the units are half as large below a power of two).  Within one unit of the
+// rounded sum.
+__device__ __forceinline__ double ff_near_to_f64(const float y, const float c)
+{
+    const int b = __float_as_int(y);
+    int k = __float2int_rn(c * __int_as_float((306 << 23) - (b & 0x7f800000)));
+    if ((b & 0x007fffff) == 0 && k < 0) k += k;
+    return __longlong_as_double(__double_as_longlong(f32_to_f64_bits(y)) + k);
+}
+
+// 1 / sqrt(a) for a > 0 in the FP32 exponent range, relative error ~2^-43, off
+// the FP64 pipe: y ~ 1/sqrt(hi) from the SFU, e = 1 - a y^2 in double-float (hi y =
+// p + p_lo exactly by an FMA), result y + y e / 2.  Falls back to the library
+// rsqrt outside that range.
 __device__ __forceinline__ double rsqrt_ff(double a)
 {
     const int hi32 = __double2hiint(a);
@@ -209,7 +229,7 @@ __device__ __forceinline__ double rsqrt_ff(double a)
     const float p_lo = fmaf(x.hi, y, -p);
     const float q = fmaf(-p, y, 1.0f);
     const float e = fmaf(-fmaf(x.lo, y, p_lo), y, q);
-    return f32_to_f64_bits(y) + f32_to_f64_signed(0.5f * y * e);
+    return ff_near_to_f64(y, 0.5f * y * e);
 }
 
 }  // namespace chs

@@ -25,6 +25,8 @@
 // hold Q (vector j, component c), rows k*d + j(j+1)/2 + i hold R_ij (i <= j).
 #include <math.h>
 
+#include <type_traits>
+
 #include "rk4_common.cuh"
 #include "seed.cuh"
 
@@ -104,21 +106,12 @@ k_init_f32(const SysPar sp, const uint64_t seed, const double* __restrict__ ics,
     for (int p = 0; p < K * (K + 1) / 2; ++p) wg[(K * D + p) * n + o] = (float)R[p];
 }
 
-// Hess V of each system (as in systems.cuh) in FP32 from the FP32-rounded stage
+// Hess V of the systems other than Henon-Heiles (whose propagator is built from the
+// stage positions, phi_build_hh) in FP32 from the FP32-rounded stage
 // positions: the frame is propagated in FP32 anyway, so forming the Hessian in
 // FP64 and rounding it would spend FP64 instructions for the same FP32 accuracy.
 template <class Sys>
 struct Hess32;
-
-template <>
-struct Hess32<SysHenonHeiles> {
-    __device__ __forceinline__ static void eval(const float* q, float* H, const SysPar&)
-    {
-        H[0] = fmaf(2.0f, q[1], 1.0f);
-        H[1] = 2.0f * q[0];
-        H[2] = fmaf(-2.0f, q[1], 1.0f);
-    }
-};
 
 template <>
 struct Hess32<SysHarmonic> {
@@ -196,12 +189,17 @@ struct FrameRun {
     __device__ __forceinline__ bool step(const StepArgs& a, const SysPar& sp)
     {
         ++s;
-        float qf[4][N], Hf[4][NH];
+        float qf[4][N];
         rk4_state_positions<Sys, LD, true>(x, L, a.dt, a.ld_sqrt, a.ld_p, sp, qf);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) Hess32<Sys>::eval(qf[q], Hf[q], sp);
         PhiBlocks<N, float> P;
-        phi_build<N, NH, float>(Hf, a.dt, P);
+        if constexpr (std::is_same<Sys, SysHenonHeiles>::value) {
+            phi_build_hh<float>(qf, a.dt, P);
+        } else {
+            float Hf[4][NH];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) Hess32<Sys>::eval(qf[q], Hf[q], sp);
+            phi_build<N, NH, float>(Hf, a.dt, P);
+        }
 #pragma unroll
         for (int j = 0; j < K; ++j) phi_apply<N, float>(P, Q[j]);
         // Phi Q = Q' S (modified Gram-Schmidt), then R <- colnorm(S R)
@@ -241,14 +239,9 @@ struct FrameRun {
 #pragma unroll
             for (int i = 0; i <= j; ++i) R[tri(i, j)] = col[i] * inv;
         }
-        if (a.escape_r2 > 0.0) {
-            double r2 = x[0] * x[0];
-#pragma unroll
-            for (int i = 1; i < N; ++i) r2 = fma(x[i], x[i], r2);
-            if (r2 > a.escape_r2) {
-                st = CHS_ORBIT_ESCAPED;
-                return false;
-            }
+        if (escaped<N>(x, a.escape_hi, a.escape_r2)) {
+            st = CHS_ORBIT_ESCAPED;
+            return false;
         }
         if (--until == 0) {
             until = a.sample_every;
@@ -320,8 +313,14 @@ __device__ __forceinline__ bool integrate_orbit_f32(const int64_t o, const StepA
 }
 
 // One thread per orbit; the orbit-selection modes of k_integrate (k_small.cu).
+// The queue form's loop keeps more registers alive; capped to the occupancy of the
+// plain form where that measured faster (262,144 orbits, 300 steps: quartic k = 4
+// 12.8 -> 11.1 ms, Henon-Heiles k = 4 without the LD 9.0 -> 5.9 ms).
 template <class Sys, int K, bool LD, int MODE>
-__global__ void __launch_bounds__(kSmallBlock)
+constexpr int kMinBlocks = MODE != kModeQueue ? 0 : Sys::N == 3 ? 3 : LD ? 0 : 4;
+
+template <class Sys, int K, bool LD, int MODE>
+__global__ void __launch_bounds__(kSmallBlock, kMinBlocks<Sys, K, LD, MODE>)
 k_integrate_f32(const StepArgs a, const SysPar sp, const EnsPtrs e, const OrbitList ol)
 {
     if constexpr (MODE == kModeQueue) {

@@ -205,7 +205,7 @@ __device__ __forceinline__ void rk4_step_phi(double* x, double (*w)[2 * Sys::N],
             q[s][0] = xs[0];
             q[s][1] = xs[1];
         });
-        phi_build_hh(q, h, P);
+        phi_build_hh<double>(q, h, P);
     } else {
         double H[4][Sys::NH];
         rk4_state_capture<Sys, LD>(x, L, h, ld_sqrt, ld_p, sp, H);
@@ -227,27 +227,6 @@ __device__ __forceinline__ void rk4_step(double* x, double (*w)[2 * Sys::N], dou
         rk4_step_phi<Sys, K, LD>(x, w, L, h, ld_sqrt, ld_p, sp);
     else
         rk4_step_direct<Sys, K, LD, double>(x, w, L, h, ld_sqrt, ld_p, sp);
-}
-
-// SALI of two vectors (each normalised first): min(|u + v|, |u - v|).
-template <int D>
-__device__ __forceinline__ double sali_of(const double* a, const double* b)
-{
-    double na = a[0] * a[0], nb = b[0] * b[0];
-#pragma unroll
-    for (int c = 1; c < D; ++c) {
-        na = fma(a[c], a[c], na);
-        nb = fma(b[c], b[c], nb);
-    }
-    const double ia = rsqrt_nr(na), ib = rsqrt_nr(nb);
-    double sp = 0.0, sm = 0.0;
-#pragma unroll
-    for (int c = 0; c < D; ++c) {
-        const double u = a[c] * ia, v = b[c] * ib;
-        sp = fma(u + v, u + v, sp);
-        sm = fma(u - v, u - v, sm);
-    }
-    return sqrt(fmin(sp, sm));
 }
 
 // The state of one orbit during a call: loaded from the ensemble, advanced
@@ -291,23 +270,11 @@ struct OrbitRun {
         rk4_step<Sys, K, LD>(x, w, L, a.dt, a.ld_sqrt, a.ld_p, sp);
         if (a.renorm) {
 #pragma unroll
-            for (int j = 0; j < K; ++j) {
-                double n2 = w[j][0] * w[j][0];
-#pragma unroll
-                for (int c = 1; c < D; ++c) n2 = fma(w[j][c], w[j][c], n2);
-                const double inv = rsqrt_ff(n2);
-#pragma unroll
-                for (int c = 0; c < D; ++c) w[j][c] *= inv;
-            }
+            for (int j = 0; j < K; ++j) unit_vector<D>(w[j]);
         }
-        if (a.escape_r2 > 0.0) {
-            double r2 = x[0] * x[0];
-#pragma unroll
-            for (int i = 1; i < N; ++i) r2 = fma(x[i], x[i], r2);
-            if (r2 > a.escape_r2) {
-                st = CHS_ORBIT_ESCAPED;
-                return false;
-            }
+        if (escaped<N>(x, a.escape_hi, a.escape_r2)) {
+            st = CHS_ORBIT_ESCAPED;
+            return false;
         }
         if (--until == 0) {
             until = a.sample_every;
@@ -538,20 +505,8 @@ k_lyap_small(const StepArgs a, const SysPar sp, const int64_t n, const double* _
 #pragma unroll
                 for (int j = 0; j < D; ++j) {
 #pragma unroll
-                    for (int i = 0; i < j; ++i) {
-                        double r = 0.0;
-#pragma unroll
-                        for (int c = 0; c < D; ++c) r = fma(W[i][c], W[j][c], r);
-#pragma unroll
-                        for (int c = 0; c < D; ++c) W[j][c] = fma(-r, W[i][c], W[j][c]);
-                    }
-                    double n2 = 0.0;
-#pragma unroll
-                    for (int c = 0; c < D; ++c) n2 = fma(W[j][c], W[j][c], n2);
-                    S[j] += 0.5 * log(n2);
-                    const double inv = rsqrt_nr(n2);
-#pragma unroll
-                    for (int c = 0; c < D; ++c) W[j][c] *= inv;
+                    for (int i = 0; i < j; ++i) remove_component<D>(W[i], W[j]);
+                    normalise_log<D>(W[j], S[j]);
                 }
             }
             if (--until == 0) {
