@@ -10,6 +10,7 @@
 
 #include <type_traits>
 
+#include "k_pipe.cuh"
 #include "rk4_common.cuh"
 #include "seed.cuh"
 
@@ -647,6 +648,7 @@ cudaError_t launch_integrate(const SysPar& sp, int k, int vec_fp32, bool ld, con
 {
     if (e.n == 0 || a.n_steps == 0) return cudaSuccess;
     if (vec_fp32 && k > 0) return launch_integrate_f32(sp, k, ld, a, e, ol, st);
+    if (pipe_applies(sp, k, a, e.n, ol)) return launch_integrate_pipe(sp, k, ld, a, e, ol, st);
     switch (sp.model) {
     case CHS_HENON_HEILES: return integ_sys<SysHenonHeiles>(k, ld, a, sp, e, ol, st);
     case CHS_HARMONIC: return integ_sys<SysHarmonic>(k, ld, a, sp, e, ol, st);
@@ -693,6 +695,7 @@ cudaError_t launch_lyap_small(const SysPar& sp, const StepArgs& a, int64_t n, co
                               cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
+    if (lyap_pipe_applies(sp, a, n)) return launch_lyap_pipe(sp, a, n, ics, ic_status, lambda, status, st);
     const unsigned g = blocks_for(n, kSmallBlock);
     switch (sp.model) {
     case CHS_HENON_HEILES:
