@@ -4,6 +4,7 @@
 // controller (safety 0.9, growth at most 10, shrink at least 0.2), every orbit
 // with its own time and step size.  Building blocks: dop853.cuh.
 #include "dop853.cuh"
+#include "k_adapt_pipe.cuh"
 
 namespace chs {
 namespace {
@@ -267,6 +268,7 @@ cudaError_t launch_integrate_adaptive(const SysPar& sp, int k, bool ld, const St
                                       cudaStream_t st)
 {
     if (e.n == 0 || a.n_steps == 0) return cudaSuccess;
+    if (adapt_pipe_applies(sp, k, ld, e.n)) return launch_adaptive_pipe(k, a, ad, e, ap, st);
     switch (sp.model) {
     case CHS_HENON_HEILES: return adapt_sys<SysHenonHeiles>(k, ld, a, ad, sp, e, ap, st);
     case CHS_HARMONIC: return adapt_sys<SysHarmonic>(k, ld, a, ad, sp, e, ap, st);
