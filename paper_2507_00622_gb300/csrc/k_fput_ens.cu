@@ -4,12 +4,8 @@
 // indicators SALI and GALI_2..k.  The paper times GALI_4 of 1e3 FPU orbits
 // against the number of degrees of freedom; this is that workload.
 //
-// A step runs in the two phases of fput_stages.cuh on the lanes of fput_ens.cuh:
-// the orbit through its stages, then every deviation vector through the same
-// stages.  With renorm the vectors are scaled to unit length inside phase 2.
-// The checks of fput_ens.cuh follow.  A warp steps its orbits in lockstep; a
-// frozen or finished orbit takes steps of size 0 (its state is not written)
-// until every orbit of the warp is done.
+// A step runs in the two phases of fput_stages.cuh, pipelined over the warps of a
+// block (fput_ens.cuh).
 #include "fput_ens.cuh"
 #include "seed.cuh"
 
@@ -80,66 +76,13 @@ k_fput_ens_init(const SysPar sp, const int K, const int renorm, const uint64_t s
 }
 
 // Fixed steps of size a.dt with the tableau Tab.
-template <int N, class Tab>
-__global__ void __launch_bounds__(32)
+template <int N, class Tab, bool PIPE>
+__global__ void __launch_bounds__(PIPE ? 32 * (1 + fe::kVecWarps) : 32)
 k_fput_ens(const StepArgs a, const SysPar sp, const int K, const EnsPtrs e)
 {
-    using C = fe::Cfg<N, Tab>;
-    constexpr int R = C::R;
     extern __shared__ double smem[];
-    const fe::Lane<N, Tab> ln(smem);
-    const int64_t o = (int64_t)blockIdx.x * C::OPW + threadIdx.x / C::L;
-    const bool valid = o < e.n;
-
-    int32_t st = valid ? e.status[o] : CHS_ORBIT_FORBIDDEN;
-    const bool runs = st == CHS_ORBIT_OK;
-    int64_t todo = 0;
-    if (runs) {
-        todo = a.n_steps;
-        if (e.t_end) {
-            const int64_t rem = e.t_end[o] - e.n_exec[o];
-            if (rem < todo) todo = rem > 0 ? rem : 0;
-        }
-    }
-    double q[R], p[R], nq[R], np[R], s5, s3;
-    ln.load(e, o, K, valid, q, p);
-    const double h0 = runs ? e.h0[o] : 0.0;
-    double dhm = runs ? e.dh_max[o] : 0.0;
-    int64_t done = 0;
-    bool active = runs && todo > 0;
-    const dp::StepH full = dp::step_h(a.dt);
-    const long long t_start = clock64();
-
-    for (int64_t it = 1;; ++it) {
-        if (!__any_sync(fe::kFull, active)) break;
-        const dp::StepH sh = active ? full : dp::StepH{0.0, 0.0, 0.0};
-        ln.template orbit_step<false>(q, p, sh, sp, nq, np, 0.0, 0.0, s5, s3);
-        ln.vectors_step(K, sh, a.renorm);
-        const bool stepped = active;
-        if (stepped) {
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                q[k] = nq[k];
-                p[k] = np[k];
-            }
-            ++done;
-        }
-        const bool check = a.sample_every > 0 && (a.step0 + it) % a.sample_every == 0;
-        st = ln.post_step(a, sp, K, q, p, stepped, check, check, h0, dhm, st);
-        if (check && a.clock_budget > 0) {  // warp-uniform: the warp's orbits stop together
-            const bool over = __any_sync(fe::kFull, budget_spent(a, t_start)) != 0;
-            if (over && stepped && st == CHS_ORBIT_OK) st = CHS_ORBIT_STEP_BUDGET;
-        }
-        active = stepped && st == CHS_ORBIT_OK && done < todo;
-    }
-    if (runs) {
-        ln.store(e, o, K, q, p);
-        if (ln.first) {
-            e.dh_max[o] = dhm;
-            e.n_exec[o] += done;
-            e.status[o] = st;
-        }
-    }
+    __shared__ fe::Ctl ctl;
+    fe::ensemble_block<N, Tab, false, PIPE>(a, AdaptArgs{}, sp, K, e, AdaptPtrs{}, smem, ctl);
 }
 
 // SALI, GALI_2..K (prod R_jj of a modified Gram-Schmidt QR of the unit
@@ -236,7 +179,9 @@ template <int N, class Tab>
 cudaError_t ens_n(const SysPar& sp, int k, const StepArgs& a, const EnsPtrs& e, cudaStream_t st)
 {
     using C = fe::Cfg<N, Tab>;
-    k_fput_ens<N, Tab><<<blocks_for(e.n, C::OPW), 32, C::smem(k), st>>>(a, sp, k, e);
+    const bool pipe = C::pipelined(k, e.n);
+    auto kern = pipe ? k_fput_ens<N, Tab, true> : k_fput_ens<N, Tab, false>;
+    kern<<<blocks_for(e.n, C::OPW), C::threads(k, pipe), C::smem(k, pipe), st>>>(a, sp, k, e);
     return cudaGetLastError();
 }
 
