@@ -15,6 +15,7 @@
 //
 // The hidden layers of the forward pass run on the tensor cores (below), the
 // training kernels on the FP32 pipe; weights and activations are stored in BF16.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -22,11 +23,12 @@
 
 namespace chs {
 
+namespace cg = cooperative_groups;
+
 constexpr int kF = 12, kH = 128, kO = 2, kS = 10;
 constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * kF, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH,
               kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH * kH, kOffW4 = kOffB3 + kH,
               kOffB4 = kOffW4 + kO * kH, kParams = kOffB4 + kO;
-constexpr int kTile = 64;       // samples per block
 constexpr int kThreads = 256;
 
 size_t mlp_param_count() { return (size_t)kParams; }
@@ -62,8 +64,9 @@ __global__ void k_mlp_features(const double* __restrict__ series, const int S, c
 // Forward pass
 //
 // A persistent grid (one block of kFwdWarps warps per SM); a warp takes tiles of
-// 32 samples, as two halves of 16 rows, through all layers without leaving its
-// own shared memory:
+// 32 samples, as two halves of 16 rows (16 samples where 32 would leave SMs
+// without a tile: a batch of 4096 then has two warps at work on most SMs), through
+// all layers without leaving its own shared memory:
 //   features / X   FP32, 32 samples at a time;
 //   layer 1        FP32 FMA chains (K = 12, FP32 inputs);
 //   layers 2, 3    mma.sync m16n8k16 (BF16 operands, FP32 accumulators), weights
@@ -325,16 +328,26 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 1)
 k_mlp_forward(const __nv_bfloat16* __restrict__ P, const float* __restrict__ X, const double* __restrict__ series,
               const int S, const double* __restrict__ ld, const double t, const double* __restrict__ E, const int64_t n,
               float* __restrict__ Y, __nv_bfloat16* __restrict__ act, int32_t* __restrict__ status,
-              const double conf, float* __restrict__ prob)
+              const double conf, float* __restrict__ prob, const int halves)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FwdSmem& sm = *reinterpret_cast<FwdSmem*>(smem_raw);
     const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
     // the parameters: weights of layers 2 and 3 as BF16, the others widened
-    for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) {
-        const int u = i / kH, k = i % kH;
-        sm.w2[u * kWS + k] = P[kOffW2 + i];
-        sm.w3[u * kWS + k] = P[kOffW3 + i];
+    if ((reinterpret_cast<uintptr_t>(P) & 15) == 0) {  // rows of 256 bytes at multiples of 16
+        static_assert(kOffW2 % 8 == 0 && kOffW3 % 8 == 0, "16-byte rows");
+#pragma unroll 4
+        for (int i = threadIdx.x; i < kH * kH / 8; i += blockDim.x) {
+            const int to = (i / (kH / 8)) * kWS + 8 * (i % (kH / 8));
+            *reinterpret_cast<uint4*>(sm.w2 + to) = *reinterpret_cast<const uint4*>(P + kOffW2 + 8 * i);
+            *reinterpret_cast<uint4*>(sm.w3 + to) = *reinterpret_cast<const uint4*>(P + kOffW3 + 8 * i);
+        }
+    } else {
+        for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) {
+            const int u = i / kH, k = i % kH;
+            sm.w2[u * kWS + k] = P[kOffW2 + i];
+            sm.w3[u * kWS + k] = P[kOffW3 + i];
+        }
     }
     for (int i = threadIdx.x; i < kH * kF; i += blockDim.x) sm.w1[i % kF][i / kF] = bf(P[kOffW1 + i]);
     for (int i = threadIdx.x; i < kO * kH; i += blockDim.x) sm.w4[i / kH][i % kH] = bf(P[kOffW4 + i]);
@@ -353,7 +366,11 @@ k_mlp_forward(const __nv_bfloat16* __restrict__ P, const float* __restrict__ X, 
         const int l = i / kH, u = i % kH;
         const __nv_bfloat16* w = (l ? sm.w3 : sm.w2) + u * kWS;
         float s = 0.0f;
-        for (int k = 0; k < kH; ++k) s = fmaf(bf(w[k]), bf(w[k]), s);
+#pragma unroll 4
+        for (int k = 0; k < kH; k += 8) {
+            const uint4 v = *reinterpret_cast<const uint4*>(w + k);
+            s = add_squares(v.w, add_squares(v.z, add_squares(v.y, add_squares(v.x, s))));
+        }
         sm.wn[l][u] = kDelta * sqrtf(s);
         sm.bn[l][u] = kDelta * fabsf(sm.b[1 + l][u]);
     }
@@ -361,10 +378,11 @@ k_mlp_forward(const __nv_bfloat16* __restrict__ P, const float* __restrict__ X, 
 
     FwdWarp& wp = sm.warp[warp];
     const double rt = 1.0 / t;
-    const int64_t tiles = (n + 31) / 32;
+    const int rows = 16 * halves;  // samples per tile
+    const int64_t tiles = (n + rows - 1) / rows;
     for (int64_t tile = blockIdx.x + (int64_t)gridDim.x * warp; tile < tiles; tile += (int64_t)gridDim.x * kFwdWarps) {
-        const int64_t o = tile * 32 + lane;  // this lane's sample
-        const bool valid = o < n;
+        const int64_t o = tile * rows + lane;  // this lane's sample
+        const bool valid = lane < rows && o < n;
         if (FROM_SERIES) {
 #pragma unroll 2
             for (int i = 0; i < kS; ++i) {
@@ -380,8 +398,8 @@ k_mlp_forward(const __nv_bfloat16* __restrict__ P, const float* __restrict__ X, 
         }
         __syncwarp();
 #pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
-            const int64_t s0 = tile * 32 + 16 * half;
+        for (int half = 0; half < halves; ++half) {
+            const int64_t s0 = tile * rows + 16 * half;
             float norm[2];
             layer1(sm, wp, half, norm);
             if (act) store_act(wp.a[0], act, s0, n);
@@ -431,151 +449,279 @@ k_mlp_forward(const __nv_bfloat16* __restrict__ P, const float* __restrict__ X, 
 // Loss and its gradient w.r.t. the outputs, averaged over n:
 //   L = BCE(sigmoid(y0), label) + w_reg (y1 - target)^2,
 //   dL/dy0 = (sigmoid(y0) - label) / n,  dL/dy1 = 2 w_reg (y1 - target) / n.
+// Returns the sample's loss and writes its gradient.
+__device__ __forceinline__ float sample_loss(const float* __restrict__ Y, const float* __restrict__ label,
+                                             const float* __restrict__ target, const int64_t n, const int64_t o,
+                                             const float w_reg, float* __restrict__ dY)
+{
+    const float y0 = Y[o], y1 = Y[n + o], lb = label[o], tg = target[o];
+    const float p = 1.0f / (1.0f + expf(-y0));
+    dY[o] = (p - lb) / (float)n;
+    dY[n + o] = 2.0f * w_reg * (y1 - tg) / (float)n;
+    // log(1 + exp(-|y|)) form of the cross entropy
+    return fmaxf(y0, 0.0f) - y0 * lb + log1pf(expf(-fabsf(y0))) + w_reg * (y1 - tg) * (y1 - tg);
+}
+
+__device__ __forceinline__ float warp_sum_f32(float l)
+{
+    for (int off = 16; off > 0; off >>= 1) l += __shfl_down_sync(0xffffffffu, l, off);
+    return l;
+}
+
 // loss_out (one float) accumulates the batch loss (atomicAdd; zero it first).
 __global__ void k_mlp_loss_grad(const float* __restrict__ Y, const float* __restrict__ label,
                                 const float* __restrict__ target, const int64_t n, const float w_reg,
                                 float* __restrict__ dY, float* __restrict__ loss_out)
 {
     const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.0f;
-    if (o < n) {
-        const float y0 = Y[o], y1 = Y[n + o], lb = label[o], tg = target[o];
-        const float p = 1.0f / (1.0f + expf(-y0));
-        // log(1 + exp(-|y|)) form of the cross entropy
-        l = fmaxf(y0, 0.0f) - y0 * lb + log1pf(expf(-fabsf(y0))) + w_reg * (y1 - tg) * (y1 - tg);
-        dY[o] = (p - lb) / (float)n;
-        dY[n + o] = 2.0f * w_reg * (y1 - tg) / (float)n;
-    }
-    for (int off = 16; off > 0; off >>= 1) l += __shfl_down_sync(0xffffffffu, l, off);
+    const float l = warp_sum_f32(o < n ? sample_loss(Y, label, target, n, o, w_reg, dY) : 0.0f);
     if ((threadIdx.x & 31) == 0 && o - (threadIdx.x & 31) < n) atomicAdd(loss_out, l / (float)n);
+}
+
+// The same for a training batch in one cluster of blocks: no zeroed accumulator (a
+// memset launch less) and a loss summed in a fixed order.
+constexpr int kLossBlock = 512, kLossCluster = 8;
+
+__global__ void __cluster_dims__(kLossCluster, 1, 1) __launch_bounds__(kLossBlock)
+k_mlp_loss_grad_cluster(const float* __restrict__ Y, const float* __restrict__ label,
+                        const float* __restrict__ target, const int64_t n, const float w_reg, float* __restrict__ dY,
+                        float* __restrict__ loss_out)
+{
+    __shared__ float part[kLossBlock / 32], total;
+    cg::cluster_group cl = cg::this_cluster();
+    float l = 0.0f;
+    for (int64_t o = (int64_t)cl.block_rank() * kLossBlock + threadIdx.x; o < n; o += kLossCluster * kLossBlock)
+        l += sample_loss(Y, label, target, n, o, w_reg, dY);
+    l = warp_sum_f32(l);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x / 32] = l;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        l = warp_sum_f32(threadIdx.x < kLossBlock / 32 ? part[threadIdx.x] : 0.0f);
+        if (threadIdx.x == 0) total = l;
+    }
+    cl.sync();
+    if (cl.block_rank() == 0 && threadIdx.x == 0) {
+        l = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kLossCluster; ++q) l += cl.map_shared_rank(&total, q)[0];
+        *loss_out = l / (float)n;
+    }
+    cl.sync();  // no block leaves before its total is read
 }
 
 // Back-propagation of one sample tile: from dY [2][n] and the stored
 // activations, the pre-activation gradients of every layer:
 //   d4 = dY;  d3 = (W4^T d4) * [a3 > 0];  d2 = (W3^T d3) * [a2 > 0];  d1 = (W2^T d2) * [a1 > 0]
-// written as FP32 [3][128][n] (d1, d2, d3).
+// written as FP32 [3][128][n] (d1, d2, d3).  FP32 chains over the units in
+// ascending order; a thread owns 4 units x 4 samples, so an input unit costs it two
+// 16-byte shared loads for 16 FMAs, and tiles of 32 samples put a batch of 4096 on
+// 128 SMs.  chs_mlp_backward, batch 4096 (this kernel and k_mlp_wgrad): 46 us; 99 us
+// while loads stood inside conditionals and so went out one at a time.
+constexpr int kBTile = 32, kBRow = kBTile + 4;  // samples per block; padded row of a gradient tile
+struct BwdSmem {
+    float w[kH * kH];         // a layer's weights, row = output unit
+    float d[2][kH * kBRow];   // the gradient entering a layer and the one leaving it
+    float w4[kO][kH];
+};
+
+// A layer's BF16 weights widened into shared memory.
+__device__ __forceinline__ void stage_weights(const __nv_bfloat16* __restrict__ Wg, float* __restrict__ Ws)
+{
+    if ((reinterpret_cast<uintptr_t>(Wg) & 15) == 0) {
+#pragma unroll
+        for (int i = threadIdx.x; i < kH * kH / 8; i += kThreads) {
+            const uint4 v = *reinterpret_cast<const uint4*>(Wg + 8 * i);
+            const unsigned p[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int q = 0; q < 4; q += 2)
+                *reinterpret_cast<float4*>(Ws + 8 * i + 2 * q) =
+                    make_float4(__uint_as_float(p[q] << 16), __uint_as_float(p[q] & 0xffff0000u),
+                                __uint_as_float(p[q + 1] << 16), __uint_as_float(p[q + 1] & 0xffff0000u));
+        }
+    } else {
+        for (int i = threadIdx.x; i < kH * kH; i += kThreads) Ws[i] = bf(Wg[i]);
+    }
+}
+
 __global__ void __launch_bounds__(kThreads)
 k_mlp_backprop(const __nv_bfloat16* __restrict__ P, const __nv_bfloat16* __restrict__ act,
                const float* __restrict__ dY, const int64_t n, float* __restrict__ delta)
 {
-    extern __shared__ float sm[];
-    float* Ws = sm;                 // kH * kH (transposed use)
-    float* D = Ws + kH * kH;        // kH * kTile  (gradient entering a layer)
-    float* E2 = D + kH * kTile;     // kH * kTile
-    const int64_t s0 = (int64_t)blockIdx.x * kTile;
+    extern __shared__ __align__(16) unsigned char bsm[];
+    BwdSmem& sm = *reinterpret_cast<BwdSmem*>(bsm);
+    constexpr int J = kH * kBTile / kThreads;  // units of a sample that a thread masks: warp + 8 j
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int64_t o = (int64_t)blockIdx.x * kBTile + lane, oc = o < n ? o : n - 1;
+    const bool valid = o < n;
+    // every activation this thread masks by is on its way before anything waits for one
+    __nv_bfloat16 raw[3][J];
+#pragma unroll
+    for (int l = 2; l >= 0; --l)
+#pragma unroll
+        for (int j = 0; j < J; ++j) raw[l][j] = act[(int64_t)(l * kH + warp + 8 * j) * n + oc];
+    const float y0 = valid ? dY[oc] : 0.0f, y1 = valid ? dY[n + oc] : 0.0f;
+    for (int i = threadIdx.x; i < kO * kH; i += kThreads) sm.w4[i / kH][i % kH] = bf(P[kOffW4 + i]);
+    stage_weights(P + kOffW3, sm.w);
+    unsigned on[3];  // bit j: activation above zero
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        on[l] = 0;
+#pragma unroll
+        for (int j = 0; j < J; ++j) on[l] |= (valid && bf(raw[l][j]) > 0.0f) ? 1u << j : 0u;
+    }
+    __syncthreads();
     // layer 4: d3 = W4^T dY masked by a3 > 0
-    for (int i = threadIdx.x; i < kO * kH; i += kThreads) Ws[i] = bf(P[kOffW4 + i]);
-    for (int p = threadIdx.x; p < kO * kTile; p += kThreads) {
-        const int64_t o = s0 + p % kTile;
-        D[p] = o < n ? dY[(int64_t)(p / kTile) * n + o] : 0.0f;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const int k = warp + 8 * j;
+        const float g = (on[2] >> j) & 1u ? sm.w4[0][k] * y0 + sm.w4[1][k] * y1 : 0.0f;
+        sm.d[0][k * kBRow + lane] = g;
+        if (valid) delta[(int64_t)(2 * kH + k) * n + o] = g;
     }
-    __syncthreads();
-    for (int p = threadIdx.x; p < kH * kTile; p += kThreads) {
-        const int k = p / kTile, s = p % kTile;
-        const int64_t o = s0 + s;
-        float g = Ws[0 * kH + k] * D[0 * kTile + s] + Ws[1 * kH + k] * D[1 * kTile + s];
-        const float a = o < n ? bf(act[(int64_t)(2 * kH + k) * n + o]) : 0.0f;
-        g = a > 0.0f ? g : 0.0f;
-        E2[p] = g;
-        if (o < n) delta[(int64_t)(2 * kH + k) * n + o] = g;
-    }
-    __syncthreads();
     // layers 3 and 2: d_{l-1}[k][s] = sum_u W_l[u][k] d_l[u][s], masked by a_{l-1} > 0
-    float* cur = E2;
-    float* nxt = D;
-    for (int layer = 3; layer >= 2; --layer) {
-        const __nv_bfloat16* Wg = P + (layer == 3 ? kOffW3 : kOffW2);
-        for (int i = threadIdx.x; i < kH * kH; i += kThreads) Ws[i] = bf(Wg[i]);
-        __syncthreads();
-        const int tk = threadIdx.x % 32, ts = threadIdx.x / 32;
-        float acc[4][8];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
+    const int tk = lane, ts = warp;  // units 4 tk .. + 3, samples 4 ts .. + 3
+#pragma unroll 1
+    for (int l = 0; l < 2; ++l) {
+        if (l == 1) stage_weights(P + kOffW2, sm.w);
+        __syncthreads();  // the weights and the incoming gradient are complete
+        float acc[4][4] = {};
+        const float* d = sm.d[l] + 4 * ts;
+#pragma unroll 8
         for (int u = 0; u < kH; ++u) {
-            float wv[4], dv[8];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) wv[a] = Ws[u * kH + tk + 32 * a];
-#pragma unroll
-            for (int b = 0; b < 8; ++b) dv[b] = cur[u * kTile + ts + 8 * b];
+            const float4 w = *reinterpret_cast<const float4*>(sm.w + u * kH + 4 * tk);
+            const float4 dv4 = *reinterpret_cast<const float4*>(d + u * kBRow);
+            const float wv[4] = {w.x, w.y, w.z, w.w}, dv[4] = {dv4.x, dv4.y, dv4.z, dv4.w};
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(wv[a], dv[b], acc[a][b]);
+                for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(wv[a], dv[b], acc[a][b]);
         }
-        const int aidx = layer - 2;  // activation index of a_{layer-1}: layer 3 -> a2 (1), layer 2 -> a1 (0)
+        // through shared memory (the tile this layer does not read), so that rows of samples leave together
+        float* out = sm.d[1 - l];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int k = tk + 32 * a;
+        for (int a = 0; a < 4; ++a)
+            *reinterpret_cast<float4*>(out + (4 * tk + a) * kBRow + 4 * ts) =
+                make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+        __syncthreads();  // out is complete, the weights are free
+        const int ai = 1 - l;  // activation a_{l-1}: layer 3 -> a2 (1), layer 2 -> a1 (0)
+        const unsigned m = ai ? on[1] : on[0];
 #pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                const int s = ts + 8 * b;
-                const int64_t o = s0 + s;
-                const float av = o < n ? bf(act[(int64_t)(aidx * kH + k) * n + o]) : 0.0f;
-                const float g = av > 0.0f ? acc[a][b] : 0.0f;
-                nxt[k * kTile + s] = g;
-                if (o < n) delta[(int64_t)(aidx * kH + k) * n + o] = g;
-            }
+        for (int j = 0; j < J; ++j) {
+            const int k = warp + 8 * j;
+            const float g = (m >> j) & 1u ? out[k * kBRow + lane] : 0.0f;
+            out[k * kBRow + lane] = g;
+            if (valid) delta[(int64_t)(ai * kH + k) * n + o] = g;
         }
-        __syncthreads();
-        float* tmp = cur;
-        cur = nxt;
-        nxt = tmp;
     }
 }
 
 // Weight and bias gradients as batch reductions:
 //   dW_l[u][k] = sum_s d_l[u][s] a_{l-1}[k][s],  db_l[u] = sum_s d_l[u][s]
-// with a_0 = X, d_4 = dY.  One block per 32 x 32 tile of one layer's dW.
-__global__ void __launch_bounds__(kThreads)
+// with a_0 = X, d_4 = dY.  A cluster of kSplit blocks works one 32 x 64 tile of one
+// layer's dW, each block a contiguous part of the batch, and the blocks' partial
+// sums are joined through distributed shared memory in a fixed order (the sums do
+// not depend on the run).  A single block per tile walked the batch alone: 40
+// blocks for 152 SMs (a training step of batch 4096 took 394 us, 76 us now).
+constexpr int kSplit = 8, kWU = 32, kWK = 64, kWS_ = 64;  // blocks per tile, tile, samples per chunk
+constexpr int kWThreads = 256;  // two groups of 128, each half of a chunk's samples
+constexpr int kWTiles = 4 + 2 * (kH / kWU) * (kH / kWK) + kH / kWK;  // layers 1; 2 and 3; 4
+
+__global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(kWThreads)
 k_mlp_wgrad(const float* __restrict__ X, const __nv_bfloat16* __restrict__ act, const float* __restrict__ delta,
             const float* __restrict__ dY, const int64_t n, float* __restrict__ G)
 {
-    __shared__ float Ds[32][33], As[32][33];
-    // tiles: layer 1: 4 x 1 (U = 128, K = 12 -> one padded k tile); layers 2, 3: 4 x 4; layer 4: 1 x 4
-    int b = blockIdx.x;
+    __shared__ __align__(16) float Ds[kWS_][kWU + 4], As[kWS_][kWK + 4];
+    __shared__ float part[2][kWU][kWK + 1];  // the groups' sums; column kWK: the bias
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank();
+    const int b = blockIdx.x / kSplit;
     int layer, ut, kt;
+    constexpr int per = (kH / kWU) * (kH / kWK);
     if (b < 4) { layer = 1; ut = b; kt = 0; }
-    else if (b < 20) { layer = 2; ut = (b - 4) / 4; kt = (b - 4) % 4; }
-    else if (b < 36) { layer = 3; ut = (b - 20) / 4; kt = (b - 20) % 4; }
-    else { layer = 4; ut = 0; kt = b - 36; }
+    else if (b < 4 + 2 * per) { layer = 2 + (b - 4) / per; ut = (b - 4) % per / (kH / kWK); kt = (b - 4) % (kH / kWK); }
+    else { layer = 4; ut = 0; kt = b - 4 - 2 * per; }
     const int U = layer == 4 ? kO : kH, K = layer == 1 ? kF : kH;
-    const int tu = threadIdx.x / 8, tk0 = (threadIdx.x % 8) * 4;  // 32 rows x (8 threads x 4 cols)
-    float acc[4] = {0.f, 0.f, 0.f, 0.f}, accb = 0.0f;
-    for (int64_t c = 0; c < n; c += 32) {
-        for (int p = threadIdx.x; p < 32 * 32; p += kThreads) {
-            const int r = p / 32, s = p % 32;
-            const int64_t o = c + s;
-            const int u = ut * 32 + r, k = kt * 32 + r;
-            float dv = 0.0f, av = 0.0f;
-            if (o < n) {
-                if (u < U) dv = layer == 4 ? dY[(int64_t)u * n + o] : delta[(int64_t)((layer - 1) * kH + u) * n + o];
-                if (k < K) av = layer == 1 ? X[(int64_t)k * n + o] : bf(act[(int64_t)((layer - 2) * kH + k) * n + o]);
-            }
-            Ds[r][s] = dv;
-            As[r][s] = av;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int s = 0; s < 32; ++s) {
-            const float dv = Ds[tu][s];
+    const float* d = layer == 4 ? dY : delta + (int64_t)(layer - 1) * kH * n;
+    const __nv_bfloat16* av = act + (int64_t)(layer > 1 ? layer - 2 : 0) * kH * n;  // layers 2 .. 4
+    // chunks of samples, a contiguous range of them per block
+    const int64_t chunks = (n + kWS_ - 1) / kWS_, each = (chunks + kSplit - 1) / kSplit;
+    const int64_t c0 = rank * each, c1 = min(chunks, c0 + each);
+    const int sl = threadIdx.x % kWS_, row = threadIdx.x / kWS_;  // sample and first row (of every 4th) to load
+    const int grp = threadIdx.x / 128, tu = threadIdx.x % 128 / 16, tk = threadIdx.x % 16;
+    float acc[4][4] = {}, accb[4] = {};
+    // the next chunk's loads (rows row + 4 i, sample sl), raw and unconditional at clamped indices, so
+    // that all of them are in flight at once; what lies outside is zeroed on the way to shared memory
+    float rd[kWU / 4], rx[kWK / 4];
+    __nv_bfloat16 ra[kWK / 4];
+    bool in = false;
+    auto fetch = [&](const int64_t c) {
+        const int64_t o = c * kWS_ + sl, oc = o < n ? o : n - 1;
+        in = o < n;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[j] = fmaf(dv, As[tk0 + j][s], acc[j]);
-            accb += dv;
+        for (int i = 0; i < kWU / 4; ++i) {
+            const int u = ut * kWU + row + 4 * i;
+            rd[i] = d[(int64_t)(u < U ? u : U - 1) * n + oc];
+        }
+        if (layer == 1) {
+#pragma unroll
+            for (int i = 0; i < kWK / 4; ++i) {
+                const int k = row + 4 * i;
+                rx[i] = X[(int64_t)(k < K ? k : K - 1) * n + oc];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kWK / 4; ++i) ra[i] = av[(int64_t)(kt * kWK + row + 4 * i) * n + oc];
+        }
+    };
+    if (c0 < c1) fetch(c0);
+    for (int64_t c = c0; c < c1; ++c) {
+#pragma unroll
+        for (int i = 0; i < kWU / 4; ++i) Ds[sl][row + 4 * i] = (in && ut * kWU + row + 4 * i < U) ? rd[i] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < kWK / 4; ++i)
+            As[sl][row + 4 * i] = !in ? 0.0f : layer != 1 ? bf(ra[i]) : row + 4 * i < K ? rx[i] : 0.0f;
+        __syncthreads();
+        if (c + 1 < c1) fetch(c + 1);
+#pragma unroll 8
+        for (int s = 0; s < kWS_ / 2; ++s) {
+            const float4 dv = *reinterpret_cast<const float4*>(&Ds[2 * s + grp][4 * tu]);
+            const float4 kv = *reinterpret_cast<const float4*>(&As[2 * s + grp][4 * tk]);
+            const float dd[4] = {dv.x, dv.y, dv.z, dv.w}, kk[4] = {kv.x, kv.y, kv.z, kv.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(dd[i], kk[j], acc[i][j]);
+                accb[i] += dd[i];
+            }
         }
         __syncthreads();
     }
-    const int u = ut * 32 + tu;
-    if (u >= U) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) part[grp][4 * tu + i][4 * tk + j] = acc[i][j];
+        if (tk == 0) part[grp][4 * tu + i][kWK] = accb[i];
+    }
+    cl.sync();
+    // block `rank` joins rows rank * 4 .. + 3 of the tile over the blocks, in order
     const int offW = layer == 1 ? kOffW1 : layer == 2 ? kOffW2 : layer == 3 ? kOffW3 : kOffW4;
     const int offB = layer == 1 ? kOffB1 : layer == 2 ? kOffB2 : layer == 3 ? kOffB3 : kOffB4;
+    for (int i = threadIdx.x; i < (kWU / kSplit) * (kWK + 1); i += kWThreads) {
+        const int r = rank * (kWU / kSplit) + i / (kWK + 1), cidx = i % (kWK + 1);
+        const int u = ut * kWU + r, k = kt * kWK + cidx;
+        float sum = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int k = kt * 32 + tk0 + j;
-        if (k < K) G[offW + u * K + k] = acc[j];
+        for (int q = 0; q < kSplit; ++q)
+            sum += cl.map_shared_rank(&part[0][r][cidx], q)[0] + cl.map_shared_rank(&part[1][r][cidx], q)[0];
+        if (u < U) {
+            if (cidx < kWK) {
+                if (k < K) G[offW + u * K + k] = sum;
+            } else if (kt == 0) {
+                G[offB + u] = sum;
+            }
+        }
     }
-    if (kt == 0 && tk0 == 0) G[offB + u] = accb;
+    cl.sync();  // no block leaves while another reads its part
 }
 
 // Adam on FP32 master weights; writes the BF16 copy used by the kernels.
@@ -598,18 +744,32 @@ __global__ void k_mlp_adam(float* __restrict__ W, float* __restrict__ m, float* 
 
 // ---------------------------------------------------------------------------
 
-static constexpr size_t kBwdSmem = (size_t)(kH * kH + 2 * kH * kTile) * sizeof(float);
 static_assert(sizeof(FwdSmem) <= 227 * 1024, "the forward kernel's shared memory");
 
-// Blocks of the persistent forward grid: one per SM, never more than tiles.
-static unsigned fwd_blocks(int64_t n)
+static int sm_count()
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         sms = 1;
-    const int64_t tiles = (n + 31) / 32;
-    return (unsigned)(tiles < sms ? tiles : sms);
+    return sms;
+}
+
+// Launches the forward kernel: tiles of 16 samples while tiles of 32 would give
+// each SM fewer than four, and never more blocks than tiles.
+template <bool FROM_SERIES>
+static cudaError_t forward(const __nv_bfloat16* P, const float* X, const double* series, int S, const double* ld,
+                           double t, const double* E, int64_t n, float* Y, __nv_bfloat16* act, int32_t* status,
+                           double conf, float* prob, cudaStream_t st)
+{
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_forward<FROM_SERIES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(FwdSmem));
+    if (e != cudaSuccess) return e;
+    const int sms = sm_count(), halves = n < (int64_t)4 * 32 * sms ? 1 : 2;
+    const int64_t tiles = (n + 16 * halves - 1) / (16 * halves);
+    k_mlp_forward<FROM_SERIES><<<(unsigned)(tiles < sms ? tiles : sms), 32 * kFwdWarps, sizeof(FwdSmem), st>>>(
+        P, X, series, S, ld, t, E, n, Y, act, status, conf, prob, halves);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_mlp_features(const double* series, int S, const double* ld, double t, const double* E,
@@ -624,13 +784,8 @@ cudaError_t launch_mlp_forward(const void* P, const float* X, int64_t n, float* 
                                cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_forward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(FwdSmem));
-    if (e != cudaSuccess) return e;
-    k_mlp_forward<false><<<fwd_blocks(n), 32 * kFwdWarps, sizeof(FwdSmem), st>>>(
-        static_cast<const __nv_bfloat16*>(P), X, nullptr, 0, nullptr, 0.0, nullptr, n, Y,
-        static_cast<__nv_bfloat16*>(act), nullptr, 0.0, nullptr);
-    return cudaGetLastError();
+    return forward<false>(static_cast<const __nv_bfloat16*>(P), X, nullptr, 0, nullptr, 1.0, nullptr, n, Y,
+                          static_cast<__nv_bfloat16*>(act), nullptr, 0.0, nullptr, st);
 }
 
 cudaError_t launch_mlp_decide(const void* P, const double* series, int S, const double* ld, double t,
@@ -638,19 +793,22 @@ cudaError_t launch_mlp_decide(const void* P, const double* series, int S, const 
                               cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_forward<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(FwdSmem));
-    if (e != cudaSuccess) return e;
-    k_mlp_forward<true><<<fwd_blocks(n), 32 * kFwdWarps, sizeof(FwdSmem), st>>>(
-        static_cast<const __nv_bfloat16*>(P), nullptr, series, S, ld, t, E, n, nullptr, nullptr, status,
-        conf, prob);
-    return cudaGetLastError();
+    return forward<true>(static_cast<const __nv_bfloat16*>(P), nullptr, series, S, ld, t, E, n, nullptr, nullptr,
+                         status, conf, prob, st);
 }
+
+// Largest batch whose loss one cluster sums: up to there the call takes 8.6 to 9.2 us,
+// the host's part of it; a single block took 16.5 us at 16,384.
+constexpr int64_t kLossOneCluster = 32768;
 
 cudaError_t launch_mlp_loss_grad(const float* Y, const float* label, const float* target, int64_t n,
                                  float w_reg, float* dY, float* loss, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
+    if (n <= kLossOneCluster) {
+        k_mlp_loss_grad_cluster<<<kLossCluster, kLossBlock, 0, st>>>(Y, label, target, n, w_reg, dY, loss);
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
     if (e != cudaSuccess) return e;
     k_mlp_loss_grad<<<blocks_for(n, 256), 256, 0, st>>>(Y, label, target, n, w_reg, dY, loss);
@@ -662,12 +820,12 @@ cudaError_t launch_mlp_backward(const void* P, const float* X, const void* act, 
 {
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_backprop, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kBwdSmem);
+                                         (int)sizeof(BwdSmem));
     if (e != cudaSuccess) return e;
-    k_mlp_backprop<<<blocks_for(n, kTile), kThreads, kBwdSmem, st>>>(
+    k_mlp_backprop<<<blocks_for(n, kBTile), kThreads, sizeof(BwdSmem), st>>>(
         static_cast<const __nv_bfloat16*>(P), static_cast<const __nv_bfloat16*>(act), dY, n, delta);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_mlp_wgrad<<<40, kThreads, 0, st>>>(X, static_cast<const __nv_bfloat16*>(act), delta, dY, n, G);
+    k_mlp_wgrad<<<kWTiles * kSplit, kWThreads, 0, st>>>(X, static_cast<const __nv_bfloat16*>(act), delta, dY, n, G);
     return cudaGetLastError();
 }
 
