@@ -39,6 +39,7 @@
 #include <math.h>
 
 #include "chs_internal.cuh"
+#include "fastmath.cuh"
 #include "fput_phi.cuh"
 
 namespace chs {
@@ -270,8 +271,7 @@ __device__ __forceinline__ void fput_lyap_lanes_block(const StepArgs& a, const S
                     }
                     const double nj = __shfl_sync(kFull, r[jm], js, L);  // |w_j|^2 from its lane
                     if (sub == js) nrm[jm] = nj;
-                    const double y = rsqrt(nj);
-                    const double inv2 = y * y;
+                    const double inv2 = rcp_full(nj);
 #pragma unroll
                     for (int m = jm; m < CPL; ++m) {
                         if (m > jm || sub > js) {

@@ -281,7 +281,7 @@ __device__ __forceinline__ void fput_lyap_block_n64(const StepArgs& a, const Sys
                 double nj = Pb[j];
 #pragma unroll
                 for (int q = 1; q < Q; ++q) nj += Pb[q * D + j];
-                const double inv_nj = 1.0 / nj;  // one division per pivot
+                const double inv_nj = rcp_full(nj);  // one reciprocal per pivot
                 if (t == j) nrm[j] = nj;
                 switch ((j >> 5) * 2 + ch) {
                 case 0: axpy<0, 0>(W, Pb, j, inv_nj, rb, lane); break;

@@ -43,6 +43,7 @@
 #include <math.h>
 
 #include "chs_internal.cuh"
+#include "fastmath.cuh"
 #include "fput_phi.cuh"
 
 namespace chs {
@@ -201,7 +202,7 @@ __device__ __forceinline__ void qr_split(double* W, double* P, double* Sv, doubl
         double nj = Pb[j];
 #pragma unroll
         for (int q = 1; q < Q; ++q) nj += Pb[q * D + j];
-        const double inv_nj = 1.0 / nj;  // one division per pivot, not per column
+        const double inv_nj = rcp_full(nj);  // one reciprocal per pivot, not per column
         if (t == j) nrm[j] = nj;
         switch (j >> 5) {
         case 0: split_axpy<N, 0>(W, Pb, j, inv_nj, w, lane); break;
@@ -265,7 +266,7 @@ __device__ __forceinline__ double qr_warp32(double* W, const int l)
             }
             const double nj = __shfl_sync(0xffffffffu, r[jm], jp);  // |w_j|^2
             if (l == j) n2 = nj;
-            const double inv_nj = 1.0 / nj;  // one division per pivot
+            const double inv_nj = rcp_full(nj);  // one reciprocal per pivot
 #pragma unroll
             for (int m = jm; m < CG; ++m) {
                 if (m > jm || p > jp) {
@@ -407,7 +408,7 @@ __device__ __forceinline__ void fput_lyap_block(const StepArgs& a, const SysPar&
                     }
                     __syncthreads();
                     if (l > j) {
-                        const double cfac = -r / red[0];
+                        const double cfac = -r * rcp_full(red[0]);
 #pragma unroll 4
                         for (int i = 0; i < D; ++i) W[i * D + l] = fma(cfac, W[i * D + j], W[i * D + l]);
                     }

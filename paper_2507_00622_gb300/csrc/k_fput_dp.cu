@@ -96,7 +96,7 @@ __device__ __forceinline__ void qr_step_split(double* slab, const int l, double&
         double nj = Pb[j];
 #pragma unroll
         for (int q = 1; q < Q; ++q) nj += Pb[q * D + j];
-        const double inv_nj = 1.0 / nj;  // one division per pivot, not per column
+        const double inv_nj = rcp_full(nj);  // one reciprocal per pivot, not per column
 #pragma unroll
         for (int m = 0; m < Q; ++m) {
             const int c = lane + 32 * m;
@@ -172,7 +172,7 @@ __device__ __forceinline__ void qr_step_split_wide(double* slab, const int t, do
         double nj = Pb[j];
 #pragma unroll
         for (int q = 1; q < Q; ++q) nj += Pb[q * D + j];
-        const double inv_nj = 1.0 / nj;  // one division per pivot, not per column
+        const double inv_nj = rcp_full(nj);  // one reciprocal per pivot, not per column
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int c = lane + 32 * (ch + 2 * u);
@@ -238,7 +238,7 @@ __device__ __forceinline__ void qr_step(double* slab, const int l, const bool mi
         }
         __syncthreads();
         if (mine && l > j) {
-            const double cfac = -r / red[0];
+            const double cfac = -r * rcp_full(red[0]);
 #pragma unroll 4
             for (int i = 0; i < D; ++i) wl[i] = fma(cfac, wj[i], wl[i]);
         }
