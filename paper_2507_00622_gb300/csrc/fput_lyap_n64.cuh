@@ -38,13 +38,12 @@ __device__ __forceinline__ void pair_sync(const int rb)
     asm volatile("bar.sync %0, 64;" ::"r"(1 + rb) : "memory");
 }
 
-// Partial dot products w_j . w_c over the rows of block rb for the groups
-// CH and CH + 2 that are not finished (m >= M0 = j / 32).
-template <int M0, int CH>
+// Partial dot products w_j . w_c over the rows of block rb for the groups A and B
+// that are to be worked whole.
+template <bool A, bool B, int CH>
 __device__ __forceinline__ void dots(const double* __restrict__ W, double* __restrict__ Pb, const int j,
                                      const int rb, const int lane)
 {
-    constexpr bool A = CH >= M0, B = CH + 2 >= M0;
     if constexpr (A || B) {
         const int r0 = 32 * rb, ca = lane + 32 * CH, cb = lane + 32 * (CH + 2);
         double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
@@ -66,35 +65,60 @@ __device__ __forceinline__ void dots(const double* __restrict__ W, double* __res
 }
 
 // w_c -= (r_c / r_j) w_j on the rows of block rb for the columns c > j of the
-// groups CH and CH + 2.
-template <int M0, int CH>
+// groups A (CH) and B (CH + 2).
+template <bool A, bool B, int CH>
 __device__ __forceinline__ void axpy(double* __restrict__ W, const double* __restrict__ Pb, const int j,
                                      const double inv_nj, const int rb, const int lane)
 {
-    constexpr bool A = CH >= M0, B = CH + 2 >= M0;
     if constexpr (A || B) {
         const int r0 = 32 * rb, ca = lane + 32 * CH, cb = lane + 32 * (CH + 2);
-        auto coef = [&](int c) {
-            double r = Pb[c];
-#pragma unroll
-            for (int q = 1; q < 4; ++q) r += Pb[q * D + c];
-            return -r * inv_nj;
-        };
-        const double fa = A ? coef(ca) : 0.0, fb = B ? coef(cb) : 0.0;
-        // a group above M0 lies wholly right of j; in group M0 only c > j moves
-        const bool wa = A && (CH > M0 || ca > j), wb = B && (CH + 2 > M0 || cb > j);
+        const double fa = A ? axpy_factor<D>(Pb, ca, inv_nj) : 0.0, fb = B ? axpy_factor<D>(Pb, cb, inv_nj) : 0.0;
 #pragma unroll 4
         for (int i = 0; i < 32; ++i) {
             const double wj = W[(r0 + i) * D + j];
             if constexpr (A) {
                 const double v = fma(fa, wj, W[(r0 + i) * D + ca]);
-                if (wa) W[(r0 + i) * D + ca] = v;
+                if (ca > j) W[(r0 + i) * D + ca] = v;
             }
             if constexpr (B) {
                 const double v = fma(fb, wj, W[(r0 + i) * D + cb]);
-                if (wb) W[(r0 + i) * D + cb] = v;
+                if (cb > j) W[(r0 + i) * D + cb] = v;
             }
         }
+    }
+}
+
+// A pivot of group M0 = j / 32: this warp's groups CH and CH + 2, the pivot's own
+// group narrow once at most 16 of its columns are left (fput_lyap_rk4.cuh).
+template <int M0, int CH>
+__device__ __forceinline__ void pivot_dots(const double* W, double* Pb, const int j, const int rb, const int lane)
+{
+    constexpr bool own = CH == M0 || CH + 2 == M0;
+    const int left = 32 * (M0 + 1) - j;
+    if (!own || left > 16) {
+        dots<(CH >= M0), (CH + 2 >= M0), CH>(W, Pb, j, rb, lane);
+    } else {
+        dots<(CH > M0), (CH + 2 > M0), CH>(W, Pb, j, rb, lane);
+        if (left > 8)
+            store_narrow<D, 16>(W, Pb + rb * D, j, 32 * M0 + 16, 32 * rb, lane);
+        else
+            store_narrow<D, 8>(W, Pb + rb * D, j, 32 * M0 + 24, 32 * rb, lane);
+    }
+}
+template <int M0, int CH>
+__device__ __forceinline__ void pivot_axpy(double* W, const double* Pb, const int j, const double inv_nj, const int rb,
+                                           const int lane)
+{
+    constexpr bool own = CH == M0 || CH + 2 == M0;
+    const int left = 32 * (M0 + 1) - j;
+    if (!own || left > 16) {
+        axpy<(CH >= M0), (CH + 2 >= M0), CH>(W, Pb, j, inv_nj, rb, lane);
+    } else {
+        axpy<(CH > M0), (CH + 2 > M0), CH>(W, Pb, j, inv_nj, rb, lane);
+        if (left > 8)
+            update_narrow<D, 16>(W, Pb, j, inv_nj, 32 * M0 + 16, 32 * rb, lane);
+        else
+            update_narrow<D, 8>(W, Pb, j, inv_nj, 32 * M0 + 24, 32 * rb, lane);
     }
 }
 
@@ -268,14 +292,14 @@ __device__ __forceinline__ void fput_lyap_block_n64(const StepArgs& a, const Sys
                 pair_sync(rb);  // rows of column j in this row block are final
                 double* Pb = qp + (j & 1) * Q * D;
                 switch ((j >> 5) * 2 + ch) {  // warp-uniform
-                case 0: dots<0, 0>(W, Pb, j, rb, lane); break;
-                case 1: dots<0, 1>(W, Pb, j, rb, lane); break;
-                case 2: dots<1, 0>(W, Pb, j, rb, lane); break;
-                case 3: dots<1, 1>(W, Pb, j, rb, lane); break;
-                case 4: dots<2, 0>(W, Pb, j, rb, lane); break;
-                case 5: dots<2, 1>(W, Pb, j, rb, lane); break;
-                case 6: dots<3, 0>(W, Pb, j, rb, lane); break;
-                default: dots<3, 1>(W, Pb, j, rb, lane); break;
+                case 0: pivot_dots<0, 0>(W, Pb, j, rb, lane); break;
+                case 1: pivot_dots<0, 1>(W, Pb, j, rb, lane); break;
+                case 2: pivot_dots<1, 0>(W, Pb, j, rb, lane); break;
+                case 3: pivot_dots<1, 1>(W, Pb, j, rb, lane); break;
+                case 4: pivot_dots<2, 0>(W, Pb, j, rb, lane); break;
+                case 5: pivot_dots<2, 1>(W, Pb, j, rb, lane); break;
+                case 6: pivot_dots<3, 0>(W, Pb, j, rb, lane); break;
+                default: pivot_dots<3, 1>(W, Pb, j, rb, lane); break;
                 }
                 __syncthreads();
                 double nj = Pb[j];
@@ -284,14 +308,14 @@ __device__ __forceinline__ void fput_lyap_block_n64(const StepArgs& a, const Sys
                 const double inv_nj = rcp_full(nj);  // one reciprocal per pivot
                 if (t == j) nrm[j] = nj;
                 switch ((j >> 5) * 2 + ch) {
-                case 0: axpy<0, 0>(W, Pb, j, inv_nj, rb, lane); break;
-                case 1: axpy<0, 1>(W, Pb, j, inv_nj, rb, lane); break;
-                case 2: axpy<1, 0>(W, Pb, j, inv_nj, rb, lane); break;
-                case 3: axpy<1, 1>(W, Pb, j, inv_nj, rb, lane); break;
-                case 4: axpy<2, 0>(W, Pb, j, inv_nj, rb, lane); break;
-                case 5: axpy<2, 1>(W, Pb, j, inv_nj, rb, lane); break;
-                case 6: axpy<3, 0>(W, Pb, j, inv_nj, rb, lane); break;
-                default: axpy<3, 1>(W, Pb, j, inv_nj, rb, lane); break;
+                case 0: pivot_axpy<0, 0>(W, Pb, j, inv_nj, rb, lane); break;
+                case 1: pivot_axpy<0, 1>(W, Pb, j, inv_nj, rb, lane); break;
+                case 2: pivot_axpy<1, 0>(W, Pb, j, inv_nj, rb, lane); break;
+                case 3: pivot_axpy<1, 1>(W, Pb, j, inv_nj, rb, lane); break;
+                case 4: pivot_axpy<2, 0>(W, Pb, j, inv_nj, rb, lane); break;
+                case 5: pivot_axpy<2, 1>(W, Pb, j, inv_nj, rb, lane); break;
+                case 6: pivot_axpy<3, 0>(W, Pb, j, inv_nj, rb, lane); break;
+                default: pivot_axpy<3, 1>(W, Pb, j, inv_nj, rb, lane); break;
                 }
             }
             __syncthreads();

@@ -45,6 +45,7 @@
 #include "chs_internal.cuh"
 #include "fastmath.cuh"
 #include "fput_phi.cuh"
+#include "gs_narrow.cuh"
 
 namespace chs {
 
@@ -122,12 +123,39 @@ __device__ __forceinline__ void apply_phi(double* __restrict__ W, const double* 
     }
 }
 
+// f = - (w_j . w_c) / |w_j|^2 from the four row blocks' partial sums.
+template <int D>
+__device__ __forceinline__ double axpy_factor(const double* __restrict__ Pb, const int c, const double inv_nj)
+{
+    double r = Pb[c];
+#pragma unroll
+    for (int q = 1; q < 4; ++q) r += Pb[q * D + c];
+    return -r * inv_nj;
+}
+
+// A row block's narrow dot products and updates at d = 128 (gs_narrow.cuh).
+template <int D, int WD>
+__device__ __forceinline__ void store_narrow(const double* __restrict__ W, double* __restrict__ Prow, const int j,
+                                             const int c0, const int r0, const int lane)
+{
+    const double s = gs::narrow_dot<32, WD, D, 1>(W + r0 * D, j, c0, lane);
+    if (lane < WD) Prow[c0 + lane] = s;
+}
+template <int D, int WD>
+__device__ __forceinline__ void update_narrow(double* __restrict__ W, const double* __restrict__ Pb, const int j,
+                                              const double inv_nj, const int c0, const int r0, const int lane)
+{
+    gs::narrow_axpy<32, WD, D, 1>(W + r0 * D, j, c0, lane, axpy_factor<D>(Pb, c0 + lane % WD, inv_nj));
+}
+
 // One pivot step of the split modified Gram-Schmidt for d = 128, for the
 // column groups m >= M0 (columns lane + 32 m; the groups below are finished:
 // M0 = j / 32).  The groups' dot products run in one block of code, sharing the
 // loads of the pivot column and giving the warp independent FMA chains; lanes
 // whose column is below j compute too but store only into sums nobody reads.
-template <int N, int M0>
+// From the 16th column of its group on the pivot's own group is worked narrow
+// (gs_narrow.cuh) and only the groups FROM > M0 here.
+template <int N, int FROM>
 __device__ __forceinline__ void split_dots(const double* __restrict__ W, double* __restrict__ Pb, const int j,
                                            const int w, const int lane)
 {
@@ -135,47 +163,78 @@ __device__ __forceinline__ void split_dots(const double* __restrict__ W, double*
     const int r0 = 32 * w;
     double a0[Q], a1[Q];
 #pragma unroll
-    for (int m = M0; m < Q; ++m) a0[m] = a1[m] = 0.0;
+    for (int m = FROM; m < Q; ++m) a0[m] = a1[m] = 0.0;
+    if constexpr (FROM < Q) {
 #pragma unroll 4
-    for (int i = 0; i < 32; i += 2) {
-        const double wj0 = W[(r0 + i) * D + j], wj1 = W[(r0 + i + 1) * D + j];
+        for (int i = 0; i < 32; i += 2) {
+            const double wj0 = W[(r0 + i) * D + j], wj1 = W[(r0 + i + 1) * D + j];
 #pragma unroll
-        for (int m = M0; m < Q; ++m) {
-            const int c = lane + 32 * m;
-            a0[m] = fma(wj0, W[(r0 + i) * D + c], a0[m]);
-            a1[m] = fma(wj1, W[(r0 + i + 1) * D + c], a1[m]);
+            for (int m = FROM; m < Q; ++m) {
+                const int c = lane + 32 * m;
+                a0[m] = fma(wj0, W[(r0 + i) * D + c], a0[m]);
+                a1[m] = fma(wj1, W[(r0 + i + 1) * D + c], a1[m]);
+            }
         }
     }
 #pragma unroll
-    for (int m = M0; m < Q; ++m) Pb[w * D + lane + 32 * m] = a0[m] + a1[m];
+    for (int m = FROM; m < Q; ++m) Pb[w * D + lane + 32 * m] = a0[m] + a1[m];
 }
 
-// The update of the columns c > j of this warp's rows, groups m >= M0.
-template <int N, int M0>
+// The update of the columns c > j of this warp's rows, groups m >= FROM.
+template <int N, int FROM>
 __device__ __forceinline__ void split_axpy(double* __restrict__ W, const double* __restrict__ Pb, const int j,
                                            const double inv_nj, const int w, const int lane)
 {
     constexpr int D = 2 * N, Q = D / 32;
-    const int r0 = 32 * w;
-    double f[Q];
+    if constexpr (FROM < Q) {
+        const int r0 = 32 * w;
+        double f[Q];
 #pragma unroll
-    for (int m = M0; m < Q; ++m) {
-        const int c = lane + 32 * m;
-        double r = Pb[c];
-#pragma unroll
-        for (int q = 1; q < Q; ++q) r += Pb[q * D + c];
-        f[m] = -r * inv_nj;
-    }
-    const bool diag_active = lane + 32 * M0 > j;  // groups above M0 lie wholly right of j
+        for (int m = FROM; m < Q; ++m) f[m] = axpy_factor<D>(Pb, lane + 32 * m, inv_nj);
+        const bool first_active = lane + 32 * FROM > j;  // the groups above FROM lie wholly right of j
 #pragma unroll 4
-    for (int i = 0; i < 32; ++i) {
-        const double wj = W[(r0 + i) * D + j];
+        for (int i = 0; i < 32; ++i) {
+            const double wj = W[(r0 + i) * D + j];
 #pragma unroll
-        for (int m = M0; m < Q; ++m) {
-            const int c = lane + 32 * m;
-            const double v = fma(f[m], wj, W[(r0 + i) * D + c]);
-            if (m > M0 || diag_active) W[(r0 + i) * D + c] = v;
+            for (int m = FROM; m < Q; ++m) {
+                const int c = lane + 32 * m;
+                const double v = fma(f[m], wj, W[(r0 + i) * D + c]);
+                if (m > FROM || first_active) W[(r0 + i) * D + c] = v;
+            }
         }
+    }
+}
+
+// A pivot of group M0: its dot products and its updates by the warp of row block w.
+template <int N, int M0>
+__device__ __forceinline__ void pivot_dots(const double* W, double* Pb, const int j, const int w, const int lane)
+{
+    constexpr int D = 2 * N;
+    const int left = 32 * (M0 + 1) - j;  // columns of the pivot's group that are left
+    if (left > 16) {
+        split_dots<N, M0>(W, Pb, j, w, lane);
+    } else {
+        split_dots<N, M0 + 1>(W, Pb, j, w, lane);
+        if (left > 8)
+            store_narrow<D, 16>(W, Pb + w * D, j, 32 * M0 + 16, 32 * w, lane);
+        else
+            store_narrow<D, 8>(W, Pb + w * D, j, 32 * M0 + 24, 32 * w, lane);
+    }
+}
+template <int N, int M0>
+__device__ __forceinline__ void pivot_axpy(double* W, const double* Pb, const int j, const double inv_nj, const int w,
+                                           const int lane)
+{
+    constexpr int D = 2 * N;
+    const int left = 32 * (M0 + 1) - j;
+    if (left > 16) {
+        split_axpy<N, M0>(W, Pb, j, inv_nj, w, lane);
+    } else {
+        split_axpy<N, M0 + 1>(W, Pb, j, inv_nj, w, lane);
+        if (left > 8)
+            update_narrow<D, 16>(W, Pb, j, inv_nj, 32 * M0 + 16, 32 * w, lane);
+        else
+            update_narrow<D, 8>(W, Pb, j, inv_nj, 32 * M0 + 24, 32 * w, lane);
     }
 }
 
@@ -193,10 +252,10 @@ __device__ __forceinline__ void qr_split(double* W, double* P, double* Sv, doubl
         __syncwarp();  // rows of column j in this warp's block are final
         double* Pb = P + (j & 1) * Q * D;
         switch (j >> 5) {  // block-uniform
-        case 0: split_dots<N, 0>(W, Pb, j, w, lane); break;
-        case 1: split_dots<N, 1>(W, Pb, j, w, lane); break;
-        case 2: split_dots<N, 2>(W, Pb, j, w, lane); break;
-        default: split_dots<N, 3>(W, Pb, j, w, lane); break;
+        case 0: pivot_dots<N, 0>(W, Pb, j, w, lane); break;
+        case 1: pivot_dots<N, 1>(W, Pb, j, w, lane); break;
+        case 2: pivot_dots<N, 2>(W, Pb, j, w, lane); break;
+        default: pivot_dots<N, 3>(W, Pb, j, w, lane); break;
         }
         __syncthreads();
         double nj = Pb[j];
@@ -205,10 +264,10 @@ __device__ __forceinline__ void qr_split(double* W, double* P, double* Sv, doubl
         const double inv_nj = rcp_full(nj);  // one reciprocal per pivot, not per column
         if (t == j) nrm[j] = nj;
         switch (j >> 5) {
-        case 0: split_axpy<N, 0>(W, Pb, j, inv_nj, w, lane); break;
-        case 1: split_axpy<N, 1>(W, Pb, j, inv_nj, w, lane); break;
-        case 2: split_axpy<N, 2>(W, Pb, j, inv_nj, w, lane); break;
-        default: split_axpy<N, 3>(W, Pb, j, inv_nj, w, lane); break;
+        case 0: pivot_axpy<N, 0>(W, Pb, j, inv_nj, w, lane); break;
+        case 1: pivot_axpy<N, 1>(W, Pb, j, inv_nj, w, lane); break;
+        case 2: pivot_axpy<N, 2>(W, Pb, j, inv_nj, w, lane); break;
+        default: pivot_axpy<N, 3>(W, Pb, j, inv_nj, w, lane); break;
         }
     }
     // the logarithms and reciprocal roots of the column norms after the loop,
@@ -266,7 +325,7 @@ __device__ __forceinline__ double qr_warp32(double* W, const int l)
             }
             const double nj = __shfl_sync(0xffffffffu, r[jm], jp);  // |w_j|^2
             if (l == j) n2 = nj;
-            const double inv_nj = rcp_full(nj);  // one reciprocal per pivot
+            const double inv_nj = 1.0 / nj;  // one division per pivot (rcp_full measured 1 % slower here)
 #pragma unroll
             for (int m = jm; m < CG; ++m) {
                 if (m > jm || p > jp) {
@@ -390,30 +449,8 @@ __device__ __forceinline__ void fput_lyap_block(const StepArgs& a, const SysPar&
 #pragma unroll 4
                 for (int i = 0; i < D; ++i) W[i * WS + l] *= inv;
             } else {
-                double n2 = 1.0;  // this thread's column's squared norm
-                for (int j = 0; j < D; ++j) {
-                    double r = 0.0;
-                    if (l >= j) {
-                        double r0 = 0.0, r1 = 0.0;
-#pragma unroll 4
-                        for (int i = 0; i < D; i += 2) {
-                            r0 = fma(W[i * D + j], W[i * D + l], r0);
-                            r1 = fma(W[(i + 1) * D + j], W[(i + 1) * D + l], r1);
-                        }
-                        r = r0 + r1;
-                    }
-                    if (l == j) {
-                        red[0] = r;
-                        n2 = r;
-                    }
-                    __syncthreads();
-                    if (l > j) {
-                        const double cfac = -r * rcp_full(red[0]);
-#pragma unroll 4
-                        for (int i = 0; i < D; ++i) W[i * D + l] = fma(cfac, W[i * D + j], W[i * D + l]);
-                    }
-                    __syncthreads();
-                }
+                static_assert(D == 64, "two warps per orbit");
+                const double n2 = gs::columns_mgs<D, D, 1>(W, red, l, true);
                 // the logarithm and reciprocal root of every column's norm after
                 // the loop, one per thread, instead of one lane's work inside
                 // every pivot step

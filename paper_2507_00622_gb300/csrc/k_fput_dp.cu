@@ -22,6 +22,7 @@
 // and the step factor for all of its threads; the columns of W advance only
 // for accepted trials.  A block loops until all of its orbits are done.
 #include "fput_stages.cuh"
+#include "gs_narrow.cuh"
 
 namespace chs {
 namespace {
@@ -220,29 +221,33 @@ __device__ __forceinline__ void qr_step(double* slab, const int l, const bool mi
     double* red = slab + Sl::CTL;
     double* wl = W + l * WS;
     double n2 = 1.0;  // squared norm of this thread's column
-    for (int j = 0; j < D; ++j) {
-        const double* wj = W + j * WS;
-        double r = 0.0;
-        if (mine && l >= j) {
-            double r0a = 0.0, r1a = 0.0;
+    if constexpr (D >= 32) {
+        n2 = gs::columns_mgs<D, 1, WS>(W, red, l, mine);
+    } else {
+        for (int j = 0; j < D; ++j) {
+            const double* wj = W + j * WS;
+            double r = 0.0;
+            if (mine && l >= j) {
+                double r0a = 0.0, r1a = 0.0;
 #pragma unroll 4
-            for (int i = 0; i < D; i += 2) {
-                r0a = fma(wj[i], wl[i], r0a);
-                r1a = fma(wj[i + 1], wl[i + 1], r1a);
+                for (int i = 0; i < D; i += 2) {
+                    r0a = fma(wj[i], wl[i], r0a);
+                    r1a = fma(wj[i + 1], wl[i + 1], r1a);
+                }
+                r = r0a + r1a;
             }
-            r = r0a + r1a;
-        }
-        if (mine && l == j) {
-            red[0] = r;
-            n2 = r;
-        }
-        __syncthreads();
-        if (mine && l > j) {
-            const double cfac = -r * rcp_full(red[0]);
+            if (mine && l == j) {
+                red[0] = r;
+                n2 = r;
+            }
+            __syncthreads();
+            if (mine && l > j) {
+                const double cfac = -r * rcp_full(red[0]);
 #pragma unroll 4
-            for (int i = 0; i < D; ++i) wl[i] = fma(cfac, wj[i], wl[i]);
+                for (int i = 0; i < D; ++i) wl[i] = fma(cfac, wj[i], wl[i]);
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
     // the logarithm and reciprocal root after the loop, one per thread, not one
     // lane's work inside every pivot step
