@@ -29,7 +29,6 @@ constexpr int kF = 12, kH = 128, kO = 2, kS = 10;
 constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * kF, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH,
               kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH * kH, kOffW4 = kOffB3 + kH,
               kOffB4 = kOffW4 + kO * kH, kParams = kOffB4 + kO;
-constexpr int kThreads = 256;
 
 size_t mlp_param_count() { return (size_t)kParams; }
 
@@ -87,12 +86,14 @@ __global__ void k_mlp_features(const double* __restrict__ series, const int S, c
 // activations are those of the chain and the result does not depend on the
 // tensor cores' summation order.
 //
-// chs_surrogate_decide on 524,288 samples (GB300): 0.41 ms, 5.80 ms with FP32 register
-// tiles for all layers and the library's log10; 88 TFLOP/s of 2 x 34,560 flops a
-// sample.  FP64 instruction slots (the features' logarithms, the sigmoid) bound it.
+// chs_surrogate_decide on 524,288 samples (GB300): 0.36 ms, 5.80 ms with FP32 register
+// tiles for all layers and the library's log10; 100 TFLOP/s of 2 x 34,560 flops a
+// sample.  Instruction issue bounds it (half of the slots; ALU and FP64 pipes a third
+// busy each, tensor pipe 15 %).
 // ---------------------------------------------------------------------------
 
-constexpr int kFwdWarps = 12;
+constexpr int kFwdWarps = 14;  // as many as shared memory holds
+constexpr int kQueue = 64;      // outputs of a half layer that its lanes share out for the chain
 constexpr int kWS = kH + 8;  // padded row of a BF16 matrix in shared memory (ldmatrix without conflicts)
 constexpr float kDelta = 9.5367431640625e-07f;  // 2^-20
 constexpr int kLogTab = 64;
@@ -101,6 +102,7 @@ struct alignas(16) FwdWarp {
     __nv_bfloat16 a[2][16 * kWS];  // activations of one half: layer input and output
     float x[kF][32];
     float y[2][32];
+    uint16_t queue[kQueue];        // outputs to compute by the chain: 128 row + unit
 };
 struct alignas(16) FwdSmem {
     __nv_bfloat16 w2[kH * kWS], w3[kH * kWS];
@@ -239,7 +241,8 @@ __device__ __forceinline__ void layer1(const FwdSmem& sm, FwdWarp& wp, const int
 // row norms of in, replaced by those of out.
 __device__ __forceinline__ void layer_mma(const __nv_bfloat16* __restrict__ W, const float* __restrict__ bias,
                                           const float* __restrict__ wn, const float* __restrict__ bn,
-                                          const __nv_bfloat16* in, __nv_bfloat16* out, float (&norm)[2])
+                                          const __nv_bfloat16* in, __nv_bfloat16* out, uint16_t* queue,
+                                          float (&norm)[2])
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     unsigned A[8][4];
@@ -279,12 +282,36 @@ __device__ __forceinline__ void layer_mma(const __nv_bfloat16* __restrict__ W, c
             }
         }
     }
-    while (again) {
-        const int i = __ffsll((long long)again) - 1;
-        again &= again - 1;
-        const int row = g + 8 * ((i >> 1) & 1), u = 8 * (i >> 2) + 2 * t + (i & 1);
+    // The flagged outputs (about six) are shared out over the lanes, so that the warp
+    // runs the chain once; where they are more than the queue holds (saturated or
+    // non-finite inputs) every lane works off its own.
+    const int mine = __popcll(again);
+    int before = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, before, off);
+        if (lane >= off) before += up;
+    }
+    const int total = __shfl_sync(0xffffffffu, before, 31);
+    before -= mine;
+    auto output = [&](const int i) { return 128 * (g + 8 * ((i >> 1) & 1)) + 8 * (i >> 2) + 2 * t + (i & 1); };
+    auto chain = [&](const int at) {
+        const int row = at >> 7, u = at & 127;
         const float v = chain128(W + u * kWS, in + row * kWS) + bias[u];
         out[row * kWS + u] = __float2bfloat16_rn(fmaxf(v, 0.0f));
+    };
+    if (total <= kQueue) {
+        for (int q = before; again; ++q) {
+            queue[q] = (uint16_t)output(__ffsll((long long)again) - 1);
+            again &= again - 1;
+        }
+        __syncwarp();  // the queue and the lanes' outputs are written
+        for (int q = lane; q < total; q += 32) chain(queue[q]);
+    } else {
+        while (again) {
+            chain(output(__ffsll((long long)again) - 1));
+            again &= again - 1;
+        }
     }
     row_norms(n2);
     norm[0] = n2[0];
@@ -403,9 +430,9 @@ k_mlp_forward(const __nv_bfloat16* __restrict__ P, const float* __restrict__ X, 
             float norm[2];
             layer1(sm, wp, half, norm);
             if (act) store_act(wp.a[0], act, s0, n);
-            layer_mma(sm.w2, sm.b[1], sm.wn[0], sm.bn[0], wp.a[0], wp.a[1], norm);
+            layer_mma(sm.w2, sm.b[1], sm.wn[0], sm.bn[0], wp.a[0], wp.a[1], wp.queue, norm);
             if (act) store_act(wp.a[1], act + (int64_t)kH * n, s0, n);
-            layer_mma(sm.w3, sm.b[2], sm.wn[1], sm.bn[1], wp.a[1], wp.a[0], norm);
+            layer_mma(sm.w3, sm.b[2], sm.wn[1], sm.bn[1], wp.a[1], wp.a[0], wp.queue, norm);
             if (act) store_act(wp.a[0], act + (int64_t)2 * kH * n, s0, n);
             // layer 4: lane (output, row), the chain over k
             const int row = lane & 15, out = lane >> 4;
@@ -513,11 +540,11 @@ k_mlp_loss_grad_cluster(const float* __restrict__ Y, const float* __restrict__ l
 // activations, the pre-activation gradients of every layer:
 //   d4 = dY;  d3 = (W4^T d4) * [a3 > 0];  d2 = (W3^T d3) * [a2 > 0];  d1 = (W2^T d2) * [a1 > 0]
 // written as FP32 [3][128][n] (d1, d2, d3).  FP32 chains over the units in
-// ascending order; a thread owns 4 units x 4 samples, so an input unit costs it two
-// 16-byte shared loads for 16 FMAs, and tiles of 32 samples put a batch of 4096 on
-// 128 SMs.  chs_mlp_backward, batch 4096 (this kernel and k_mlp_wgrad): 46 us; 99 us
+// ascending order; a thread owns 4 units x 2 samples, and tiles of 32 samples put a
+// batch of 4096 on 128 SMs with 16 warps each.  chs_mlp_backward, batch 4096 (this kernel and k_mlp_wgrad): 43 us; 99 us
 // while loads stood inside conditionals and so went out one at a time.
 constexpr int kBTile = 32, kBRow = kBTile + 4;  // samples per block; padded row of a gradient tile
+constexpr int kBThreads = 512;
 struct BwdSmem {
     float w[kH * kH];         // a layer's weights, row = output unit
     float d[2][kH * kBRow];   // the gradient entering a layer and the one leaving it
@@ -529,7 +556,7 @@ __device__ __forceinline__ void stage_weights(const __nv_bfloat16* __restrict__ 
 {
     if ((reinterpret_cast<uintptr_t>(Wg) & 15) == 0) {
 #pragma unroll
-        for (int i = threadIdx.x; i < kH * kH / 8; i += kThreads) {
+        for (int i = threadIdx.x; i < kH * kH / 8; i += kBThreads) {
             const uint4 v = *reinterpret_cast<const uint4*>(Wg + 8 * i);
             const unsigned p[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -539,17 +566,17 @@ __device__ __forceinline__ void stage_weights(const __nv_bfloat16* __restrict__ 
                                 __uint_as_float(p[q + 1] << 16), __uint_as_float(p[q + 1] & 0xffff0000u));
         }
     } else {
-        for (int i = threadIdx.x; i < kH * kH; i += kThreads) Ws[i] = bf(Wg[i]);
+        for (int i = threadIdx.x; i < kH * kH; i += kBThreads) Ws[i] = bf(Wg[i]);
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kBThreads)
 k_mlp_backprop(const __nv_bfloat16* __restrict__ P, const __nv_bfloat16* __restrict__ act,
                const float* __restrict__ dY, const int64_t n, float* __restrict__ delta)
 {
     extern __shared__ __align__(16) unsigned char bsm[];
     BwdSmem& sm = *reinterpret_cast<BwdSmem*>(bsm);
-    constexpr int J = kH * kBTile / kThreads;  // units of a sample that a thread masks: warp + 8 j
+    constexpr int J = kH * kBTile / kBThreads;  // units of a sample that a thread masks: warp + 16 j
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
     const int64_t o = (int64_t)blockIdx.x * kBTile + lane, oc = o < n ? o : n - 1;
     const bool valid = o < n;
@@ -558,9 +585,9 @@ k_mlp_backprop(const __nv_bfloat16* __restrict__ P, const __nv_bfloat16* __restr
 #pragma unroll
     for (int l = 2; l >= 0; --l)
 #pragma unroll
-        for (int j = 0; j < J; ++j) raw[l][j] = act[(int64_t)(l * kH + warp + 8 * j) * n + oc];
+        for (int j = 0; j < J; ++j) raw[l][j] = act[(int64_t)(l * kH + warp + 16 * j) * n + oc];
     const float y0 = valid ? dY[oc] : 0.0f, y1 = valid ? dY[n + oc] : 0.0f;
-    for (int i = threadIdx.x; i < kO * kH; i += kThreads) sm.w4[i / kH][i % kH] = bf(P[kOffW4 + i]);
+    for (int i = threadIdx.x; i < kO * kH; i += kBThreads) sm.w4[i / kH][i % kH] = bf(P[kOffW4 + i]);
     stage_weights(P + kOffW3, sm.w);
     unsigned on[3];  // bit j: activation above zero
 #pragma unroll
@@ -573,41 +600,40 @@ k_mlp_backprop(const __nv_bfloat16* __restrict__ P, const __nv_bfloat16* __restr
     // layer 4: d3 = W4^T dY masked by a3 > 0
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const int k = warp + 8 * j;
+        const int k = warp + 16 * j;
         const float g = (on[2] >> j) & 1u ? sm.w4[0][k] * y0 + sm.w4[1][k] * y1 : 0.0f;
         sm.d[0][k * kBRow + lane] = g;
         if (valid) delta[(int64_t)(2 * kH + k) * n + o] = g;
     }
     // layers 3 and 2: d_{l-1}[k][s] = sum_u W_l[u][k] d_l[u][s], masked by a_{l-1} > 0
-    const int tk = lane, ts = warp;  // units 4 tk .. + 3, samples 4 ts .. + 3
+    const int tk = lane, ts = warp;  // units 4 tk .. + 3, samples 2 ts, 2 ts + 1
 #pragma unroll 1
     for (int l = 0; l < 2; ++l) {
         if (l == 1) stage_weights(P + kOffW2, sm.w);
         __syncthreads();  // the weights and the incoming gradient are complete
-        float acc[4][4] = {};
-        const float* d = sm.d[l] + 4 * ts;
+        float acc[4][2] = {};
+        const float* d = sm.d[l] + 2 * ts;
 #pragma unroll 8
         for (int u = 0; u < kH; ++u) {
             const float4 w = *reinterpret_cast<const float4*>(sm.w + u * kH + 4 * tk);
-            const float4 dv4 = *reinterpret_cast<const float4*>(d + u * kBRow);
-            const float wv[4] = {w.x, w.y, w.z, w.w}, dv[4] = {dv4.x, dv4.y, dv4.z, dv4.w};
+            const float2 dv2 = *reinterpret_cast<const float2*>(d + u * kBRow);
+            const float wv[4] = {w.x, w.y, w.z, w.w}, dv[2] = {dv2.x, dv2.y};
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(wv[a], dv[b], acc[a][b]);
+                for (int b = 0; b < 2; ++b) acc[a][b] = fmaf(wv[a], dv[b], acc[a][b]);
         }
         // through shared memory (the tile this layer does not read), so that rows of samples leave together
         float* out = sm.d[1 - l];
 #pragma unroll
         for (int a = 0; a < 4; ++a)
-            *reinterpret_cast<float4*>(out + (4 * tk + a) * kBRow + 4 * ts) =
-                make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+            *reinterpret_cast<float2*>(out + (4 * tk + a) * kBRow + 2 * ts) = make_float2(acc[a][0], acc[a][1]);
         __syncthreads();  // out is complete, the weights are free
         const int ai = 1 - l;  // activation a_{l-1}: layer 3 -> a2 (1), layer 2 -> a1 (0)
         const unsigned m = ai ? on[1] : on[0];
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const int k = warp + 8 * j;
+            const int k = warp + 16 * j;
             const float g = (m >> j) & 1u ? out[k * kBRow + lane] : 0.0f;
             out[k * kBRow + lane] = g;
             if (valid) delta[(int64_t)(ai * kH + k) * n + o] = g;
@@ -617,12 +643,13 @@ k_mlp_backprop(const __nv_bfloat16* __restrict__ P, const __nv_bfloat16* __restr
 
 // Weight and bias gradients as batch reductions:
 //   dW_l[u][k] = sum_s d_l[u][s] a_{l-1}[k][s],  db_l[u] = sum_s d_l[u][s]
-// with a_0 = X, d_4 = dY.  A cluster of kSplit blocks works one 32 x 64 tile of one
+// with a_0 = X, d_4 = dY.  A cluster of kSplit blocks (132 blocks in all, one wave)
+// works one 32 x 64 tile of one
 // layer's dW, each block a contiguous part of the batch, and the blocks' partial
 // sums are joined through distributed shared memory in a fixed order (the sums do
 // not depend on the run).  A single block per tile walked the batch alone: 40
-// blocks for 152 SMs (a training step of batch 4096 took 394 us, 76 us now).
-constexpr int kSplit = 8, kWU = 32, kWK = 64, kWS_ = 64;  // blocks per tile, tile, samples per chunk
+// blocks for 152 SMs (a training step of batch 4096 took 394 us, 68 us now).
+constexpr int kSplit = 6, kWU = 32, kWK = 64, kWS_ = 64;  // blocks per tile, tile, samples per chunk
 constexpr int kWThreads = 256;  // two groups of 128, each half of a chunk's samples
 constexpr int kWTiles = 4 + 2 * (kH / kWU) * (kH / kWK) + kH / kWK;  // layers 1; 2 and 3; 4
 
@@ -631,7 +658,8 @@ k_mlp_wgrad(const float* __restrict__ X, const __nv_bfloat16* __restrict__ act, 
             const float* __restrict__ dY, const int64_t n, float* __restrict__ G)
 {
     __shared__ __align__(16) float Ds[kWS_][kWU + 4], As[kWS_][kWK + 4];
-    __shared__ float part[2][kWU][kWK + 1];  // the groups' sums; column kWK: the bias
+    __shared__ float part[2][kWU][kWK];  // the groups' sums
+    __shared__ float bias[2][kWU];       // of the chunks' first and second 32 samples
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int b = blockIdx.x / kSplit;
@@ -648,7 +676,7 @@ k_mlp_wgrad(const float* __restrict__ X, const __nv_bfloat16* __restrict__ act, 
     const int64_t c0 = rank * each, c1 = min(chunks, c0 + each);
     const int sl = threadIdx.x % kWS_, row = threadIdx.x / kWS_;  // sample and first row (of every 4th) to load
     const int grp = threadIdx.x / 128, tu = threadIdx.x % 128 / 16, tk = threadIdx.x % 16;
-    float acc[4][4] = {}, accb[4] = {};
+    float acc[4][4] = {}, accb[kWU / 4] = {};
     // the next chunk's loads (rows row + 4 i, sample sl), raw and unconditional at clamped indices, so
     // that all of them are in flight at once; what lies outside is zeroed on the way to shared memory
     float rd[kWU / 4], rx[kWK / 4];
@@ -676,7 +704,11 @@ k_mlp_wgrad(const float* __restrict__ X, const __nv_bfloat16* __restrict__ act, 
     if (c0 < c1) fetch(c0);
     for (int64_t c = c0; c < c1; ++c) {
 #pragma unroll
-        for (int i = 0; i < kWU / 4; ++i) Ds[sl][row + 4 * i] = (in && ut * kWU + row + 4 * i < U) ? rd[i] : 0.0f;
+        for (int i = 0; i < kWU / 4; ++i) {
+            const float v = (in && ut * kWU + row + 4 * i < U) ? rd[i] : 0.0f;
+            Ds[sl][row + 4 * i] = v;
+            accb[i] += v;
+        }
 #pragma unroll
         for (int i = 0; i < kWK / 4; ++i)
             As[sl][row + 4 * i] = !in ? 0.0f : layer != 1 ? bf(ra[i]) : row + 4 * i < K ? rx[i] : 0.0f;
@@ -688,38 +720,36 @@ k_mlp_wgrad(const float* __restrict__ X, const __nv_bfloat16* __restrict__ act, 
             const float4 kv = *reinterpret_cast<const float4*>(&As[2 * s + grp][4 * tk]);
             const float dd[4] = {dv.x, dv.y, dv.z, dv.w}, kk[4] = {kv.x, kv.y, kv.z, kv.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(dd[i], kk[j], acc[i][j]);
-                accb[i] += dd[i];
-            }
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) part[grp][4 * tu + i][4 * tk + j] = acc[i][j];
-        if (tk == 0) part[grp][4 * tu + i][kWK] = accb[i];
+#pragma unroll
+    for (int i = 0; i < kWU / 4; ++i) {  // a warp holds 32 samples of a row
+        const float v = warp_sum_f32(accb[i]);
+        if (sl % 32 == 0) bias[sl / 32][row + 4 * i] = v;
     }
     cl.sync();
-    // block `rank` joins rows rank * 4 .. + 3 of the tile over the blocks, in order
+    // the cluster's blocks share out the tile's sums and join each over the blocks, in order
     const int offW = layer == 1 ? kOffW1 : layer == 2 ? kOffW2 : layer == 3 ? kOffW3 : kOffW4;
     const int offB = layer == 1 ? kOffB1 : layer == 2 ? kOffB2 : layer == 3 ? kOffB3 : kOffB4;
-    for (int i = threadIdx.x; i < (kWU / kSplit) * (kWK + 1); i += kWThreads) {
-        const int r = rank * (kWU / kSplit) + i / (kWK + 1), cidx = i % (kWK + 1);
-        const int u = ut * kWU + r, k = kt * kWK + cidx;
+    for (int i = rank * kWThreads + threadIdx.x; i < kWU * (kWK + 1); i += kSplit * kWThreads) {
+        const bool weight = i < kWU * kWK;
+        const int r = weight ? i / kWK : i - kWU * kWK, c = weight ? i % kWK : 0;
+        const int u = ut * kWU + r, k = kt * kWK + c;
+        float* p0 = weight ? &part[0][r][c] : &bias[0][r];
+        float* p1 = weight ? &part[1][r][c] : &bias[1][r];
         float sum = 0.0f;
 #pragma unroll
-        for (int q = 0; q < kSplit; ++q)
-            sum += cl.map_shared_rank(&part[0][r][cidx], q)[0] + cl.map_shared_rank(&part[1][r][cidx], q)[0];
-        if (u < U) {
-            if (cidx < kWK) {
-                if (k < K) G[offW + u * K + k] = sum;
-            } else if (kt == 0) {
-                G[offB + u] = sum;
-            }
-        }
+        for (int q = 0; q < kSplit; ++q) sum += cl.map_shared_rank(p0, q)[0] + cl.map_shared_rank(p1, q)[0];
+        if (u < U && weight && k < K) G[offW + u * K + k] = sum;
+        if (u < U && !weight && kt == 0) G[offB + u] = sum;
     }
     cl.sync();  // no block leaves while another reads its part
 }
@@ -822,7 +852,7 @@ cudaError_t launch_mlp_backward(const void* P, const float* X, const void* act, 
     cudaError_t e = cudaFuncSetAttribute(k_mlp_backprop, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(BwdSmem));
     if (e != cudaSuccess) return e;
-    k_mlp_backprop<<<blocks_for(n, kBTile), kThreads, sizeof(BwdSmem), st>>>(
+    k_mlp_backprop<<<blocks_for(n, kBTile), kBThreads, sizeof(BwdSmem), st>>>(
         static_cast<const __nv_bfloat16*>(P), static_cast<const __nv_bfloat16*>(act), dY, n, delta);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_mlp_wgrad<<<kWTiles * kSplit, kWThreads, 0, st>>>(X, static_cast<const __nv_bfloat16*>(act), delta, dY, n, G);
