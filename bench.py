@@ -459,7 +459,7 @@ def run_mlp(args):
     fused forward pass (chs_mlp_forward) and the decision (chs_surrogate_decide:
     features, forward, status update), timed with CUDA events (best of 5 after a
     warm-up), with their multiply-add rate against the measured FP32 FMA peak
-    (the perceptron runs on the FP32 pipe with BF16 operands)."""
+    (BF16 operands; the hidden layers run on the tensor cores, so the fraction can exceed 1)."""
     import torch
 
     from paper_2507_00622_gb300 import build as cuda_build

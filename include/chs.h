@@ -258,7 +258,9 @@ chs_status chs_ensemble_init(chs_system s, const chs_params* p, const chs_ensemb
  * An orbit with t_end stops after t_end[o] total steps.  Splitting a run into
  * calls with consecutive step0 gives bit-identical results.  p->block_threads sets the
  * block size of the RK4 one-orbit-per-thread kernels (both vector precisions;
- * default 128); the DOP853 and FPUT kernels keep their own.  Supported: HENON_HEILES, HARMONIC, INVERTED
+ * default 128, but Henon-Heiles ensembles with FP64 vectors too small to fill the
+ * GPU then spread each orbit's step over the warps of a block, with the same
+ * results); the DOP853 and FPUT kernels keep their own.  Supported: HENON_HEILES, HARMONIC, INVERTED
  * (k <= 4), QUARTIC3 (k <= 6) and FPUT (N in {4, 8, 16, 32, 64}, k <= 6, FP64
  * vectors, no LD; the vectors advance through the same Runge-Kutta stages as
  * the chain, with the tridiagonal Hessian of Eq. ham_eqs_FPU). */

@@ -220,25 +220,74 @@ constexpr size_t slab_bytes()
     return (size_t)(12 * Sys::NH + K * 2 * Sys::N) * kBlock * sizeof(double);
 }
 
-// Phase 1, the orbit's twelve stages from x = (q, p) in Nystrom form:
-//   xn = the step's end point,
-//   dL = |h| sum_s b_s g_s  (g the LD integrand of f_s = (p_s, F_s); the LD grows
-//        with |t|), with h p_s = h p + sum_j a_sj G_j formed only at the stages
-//        with b_s != 0,
-// the stage matrices -h^2 Hess V into the slab, and with ERR the error sums
-// times h: h err5_q = sum_k (e5 A)_k G_k, h err5_p = (1/h) sum_s e5_s G_s, and err3
-// likewise.  The small terms are summed first and added to the state last.
-template <class Sys, bool LD, bool ERR>
+// The LD of a step, dL = |h| sum_s b_s g_s with g the LD integrand of f_s = (p_s, F_s)
+// (the LD grows with |t|): stage s's part, from h p and the stages' G, with h p_s = h p
+// + sum_j a_sj G_j formed only at the stages with b_s != 0.  p = 1/2: sums of
+// sqrt|h p_s| and of sqrt|h^2 F_s| in double-float, widened once per stage; their
+// factors |h|^(-1/2) and 1/|h| are applied at the end of the step (ld_total).
+struct LdSum {
+    double g = 0.0, gq = 0.0;
+};
+template <class Sys, int s>
+__device__ __forceinline__ void ld_stage(const double* hp, const double (*G)[Sys::N], const StepH sh,
+                                         const int ld_sqrt, const double ld_p, LdSum& sum)
+{
+    constexpr int N = Sys::N;
+    constexpr double cb = kB[s];
+    if constexpr (cb != 0.0) {
+        double hps[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            hps[i] = hp[i];
+            static_for<0, s>([&](auto jc) {
+                constexpr int j = decltype(jc)::value;
+                constexpr double c = kA[s][j];
+                if constexpr (c != 0.0) hps[i] = fma(c, G[j][i], hps[i]);
+            });
+        }
+        if (ld_sqrt) {
+            sum.gq = fma(cb, ff_to_f64(ff_sum_sqrt_abs<N>(hps)), sum.gq);
+            sum.g = fma(cb, ff_to_f64(ff_sum_sqrt_abs<N>(G[s])), sum.g);
+        } else {
+            double f[2 * N];
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                f[i] = sh.rh * hps[i];
+                f[N + i] = sh.rh * (sh.rh * G[s][i]);
+            }
+            sum.g = fma(cb, ld_integrand_pow<2 * N>(f, ld_p), sum.g);
+        }
+    }
+}
+__device__ __forceinline__ double ld_total(const StepH sh, const int ld_sqrt, const LdSum& sum)
+{
+    return ld_sqrt ? fma(sqrt(fabs(sh.h)), sum.gq, sum.g) : fabs(sh.h) * sum.g;
+}
+
+// For callers of orbit_step that have no use for the stages' G.
+struct KeepNothing {
+    template <class... T>
+    __device__ __forceinline__ void operator()(T...) const
+    {
+    }
+};
+
+// Phase 1, the orbit's twelve stages from x = (q, p) in Nystrom form: xn = the
+// step's end point, dL the LD of the step, the stage matrices -h^2 Hess V into the
+// slab, and with ERR the error sums times h: h err5_q = sum_k (e5 A)_k G_k, h err5_p =
+// (1/h) sum_s e5_s G_s, and err3 likewise.  The small terms are summed first and
+// added to the state last.  keep(s, G_s) is called for every stage.
+template <class Sys, bool LD, bool ERR, class Keep = KeepNothing>
 __device__ __forceinline__ void orbit_step(const Slab<Sys>& sl, const double* x, const StepH sh,
                                            const int ld_sqrt, const double ld_p, const SysPar& sp,
-                                           double* xn, double& dL, double* e5, double* e3)
+                                           double* xn, double& dL, double* e5, double* e3, Keep keep = Keep{})
 {
     constexpr int N = Sys::N, NH = Sys::NH;
     double G[12][N], hp[N], sq[N], sv[N], q5[N], q3[N], p5[N], p3[N];
-    double sL = 0.0, sLq = 0.0;
+    LdSum ld;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-        hp[i] = sh.h * x[N + i];
+        hp[i] = __dmul_rn(sh.h, x[N + i]);
         sq[i] = sv[i] = q5[i] = q3[i] = p5[i] = p3[i] = 0.0;
     }
     static_for<0, 12>([&](auto sc) {
@@ -250,6 +299,7 @@ __device__ __forceinline__ void orbit_step(const Slab<Sys>& sl, const double* x,
         Sys::eval_scaled(qs, sh.nh2, G[s], H, sp);
 #pragma unroll
         for (int t = 0; t < NH; ++t) sl.H(s, t) = H[t];
+        keep(s, G[s]);
         constexpr double cb = kB[s], nb = kNb<s>;
 #pragma unroll
         for (int i = 0; i < N; ++i) {
@@ -263,32 +313,7 @@ __device__ __forceinline__ void orbit_step(const Slab<Sys>& sl, const double* x,
                 if constexpr (c3 != 0.0) p3[i] = fma(c3, G[s][i], p3[i]);
             }
         }
-        if constexpr (LD && cb != 0.0) {
-            double hps[N];
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-                hps[i] = hp[i];
-                static_for<0, s>([&](auto jc) {
-                    constexpr int j = decltype(jc)::value;
-                    constexpr double c = kA[s][j];
-                    if constexpr (c != 0.0) hps[i] = fma(c, G[j][i], hps[i]);
-                });
-            }
-            if (ld_sqrt) {
-                // p = 1/2: sums of sqrt|h p_s| and of sqrt|h^2 F_s| in double-float, widened once;
-                // their factors |h|^(-1/2) and 1/|h| are applied at the end of the step
-                sLq = fma(cb, ff_to_f64(ff_sum_sqrt_abs<N>(hps)), sLq);
-                sL = fma(cb, ff_to_f64(ff_sum_sqrt_abs<N>(G[s])), sL);
-            } else {
-                double f[2 * N];
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    f[i] = sh.rh * hps[i];
-                    f[N + i] = sh.rh * (sh.rh * G[s][i]);
-                }
-                sL = fma(cb, ld_integrand_pow<2 * N>(f, ld_p), sL);
-            }
-        }
+        if constexpr (LD) ld_stage<Sys, s>(hp, G, sh, ld_sqrt, ld_p, ld);
     });
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -301,7 +326,7 @@ __device__ __forceinline__ void orbit_step(const Slab<Sys>& sl, const double* x,
             e3[N + i] = sh.rh * p3[i];
         }
     }
-    if constexpr (LD) dL = ld_sqrt ? fma(sqrt(fabs(sh.h)), sLq, sL) : fabs(sh.h) * sL;
+    if constexpr (LD) dL = ld_total(sh, ld_sqrt, ld);
 }
 
 // Phase 2, one deviation vector w = (u, v) through the twelve stages of
@@ -316,7 +341,7 @@ __device__ __forceinline__ void vector_step(const Slab<Sys>& sl, double* w, cons
     double G[12][N], hv[N], sq[N], sv[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-        hv[i] = sh.h * w[N + i];
+        hv[i] = __dmul_rn(sh.h, w[N + i]);
         sq[i] = sv[i] = 0.0;
     }
     static_for<0, 12>([&](auto sc) {
@@ -412,15 +437,9 @@ __device__ __forceinline__ void vectors_step(const Slab<Sys>& sl, const StepH sh
 #pragma unroll
         for (int c = 0; c < D; ++c) w[c] = sl.W(j, c);
         vector_step<Sys>(sl, w, sh);
-        double inv = 1.0;
-        if (renorm) {
-            double n2 = w[0] * w[0];
+        if (renorm) unit_vector<D>(w);
 #pragma unroll
-            for (int c = 1; c < D; ++c) n2 = fma(w[c], w[c], n2);
-            inv = rsqrt_ff(n2);
-        }
-#pragma unroll
-        for (int c = 0; c < D; ++c) sl.W(j, c) = w[c] * inv;
+        for (int c = 0; c < D; ++c) sl.W(j, c) = w[c];
     }
 }
 

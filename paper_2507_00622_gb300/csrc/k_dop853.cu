@@ -7,6 +7,7 @@
 // dop853.cuh.
 #include "k_dop853.cuh"
 #include "k_dop853_fixed.cuh"
+#include "k_dp_pipe.cuh"
 
 namespace chs {
 namespace {
@@ -97,6 +98,7 @@ cudaError_t launch_integrate_dp(const SysPar& sp, int k, bool ld, const StepArgs
                                 const EnsPtrs& e, const OrbitList* ol, cudaStream_t st)
 {
     if (e.n == 0 || a.n_steps == 0) return cudaSuccess;
+    if (dp_pipe_applies(sp, k, ld, a, e.n)) return launch_dp_pipe(sp, k, ld, a, e, ol, st);
     switch (sp.model) {
     case CHS_HENON_HEILES: return fixed_sys<SysHenonHeiles>(k, ld, a, sp, e, ol, st);
     case CHS_HARMONIC: return fixed_sys<SysHarmonic>(k, ld, a, sp, e, ol, st);

@@ -390,7 +390,7 @@ cudaError_t pipe_k(const StepArgs& a, const SysPar& sp, const EnsPtrs& e, const 
 {
     const unsigned g = blocks_for(e.n, 32);
     constexpr int threads = 32 * PipeCfg<K, LD>::WARPS;
-    if (ol)
+    if (ol && ol->list)
         k_integrate_pipe<K, LD, kModeList><<<g, threads, 0, st>>>(a, sp, e, *ol);
     else
         k_integrate_pipe<K, LD, kModeAll><<<g, threads, 0, st>>>(a, sp, e, OrbitList{});
@@ -417,10 +417,11 @@ cudaError_t pipe_ld(int k, const StepArgs& a, const SysPar& sp, const EnsPtrs& e
 // SM the GPU is full either way.
 // It is drained at every health check (two of its iterations), which at
 // intervals below 16 steps costs more than an eighth.  A block size that the
-// caller asked for runs the one-thread form; queue launches do as well.
-bool pipe_applies(const SysPar& sp, int k, const StepArgs& a, int64_t n, const OrbitList* ol)
+// caller asked for runs the one-thread form.  A queue launch of so few orbits, which
+// hold every warp at once anyway, runs it without the queue.
+bool pipe_applies(const SysPar& sp, int k, const StepArgs& a, int64_t n)
 {
-    return sp.model == CHS_HENON_HEILES && k >= 2 && k <= 4 && a.block == 0 && (!ol || !ol->queue) &&
+    return sp.model == CHS_HENON_HEILES && k >= 2 && k <= 4 && a.block == 0 &&
            (a.sample_every == 0 || a.sample_every >= 16) && n <= kPipeOrbits;
 }
 

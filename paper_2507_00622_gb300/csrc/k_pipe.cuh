@@ -9,7 +9,7 @@ namespace chs {
 constexpr int64_t kPipeOrbits = 14592;
 
 // Whether an RK4 run with FP64 vectors takes the pipelined form.
-bool pipe_applies(const SysPar& sp, int k, const StepArgs& a, int64_t n, const OrbitList* ol);
+bool pipe_applies(const SysPar& sp, int k, const StepArgs& a, int64_t n);
 cudaError_t launch_integrate_pipe(const SysPar& sp, int k, bool ld, const StepArgs& a, const EnsPtrs& e,
                                   const OrbitList* ol, cudaStream_t st);
 

@@ -648,7 +648,7 @@ cudaError_t launch_integrate(const SysPar& sp, int k, int vec_fp32, bool ld, con
 {
     if (e.n == 0 || a.n_steps == 0) return cudaSuccess;
     if (vec_fp32 && k > 0) return launch_integrate_f32(sp, k, ld, a, e, ol, st);
-    if (pipe_applies(sp, k, a, e.n, ol)) return launch_integrate_pipe(sp, k, ld, a, e, ol, st);
+    if (pipe_applies(sp, k, a, e.n)) return launch_integrate_pipe(sp, k, ld, a, e, ol, st);
     switch (sp.model) {
     case CHS_HENON_HEILES: return integ_sys<SysHenonHeiles>(k, ld, a, sp, e, ol, st);
     case CHS_HARMONIC: return integ_sys<SysHarmonic>(k, ld, a, sp, e, ol, st);

@@ -41,6 +41,8 @@ def _run(n, k, block, steps, launch="batch", splits=1, t_end=None, w_in=None, **
         prm = chs.params(dt, steps // splits, step0=i * (steps // splits), **par)
         if launch == "compacted":
             chs.chs_integrate_compacted(S.h, prm, abi, 23, work)
+        elif launch == "persistent":
+            chs.chs_integrate_persistent(S.h, prm, abi, work)
         else:
             chs.chs_integrate_batch(S.h, prm, abi)
     torch.cuda.synchronize()
@@ -71,6 +73,7 @@ def test_pipeline_uneven_ends_resume_and_lists():
     _same(a, _run(n, k, 0, 240, t_end=t_end, **kw))
     _same(a, _run(n, k, 0, 240, splits=5, t_end=t_end, **kw))
     _same(a, _run(n, k, 0, 240, launch="compacted", t_end=t_end, **kw))
+    _same(a, _run(n, k, 0, 240, launch="persistent", t_end=t_end, **kw))
 
 
 @pytest.mark.parametrize("kw", [dict(sample_every=0), dict(sample_every=16, dh_limit=2e-11),
