@@ -307,7 +307,8 @@ chs_status chs_integrate_adaptive(chs_system s, const chs_params* p, const chs_a
                                   double* err_max, int64_t* n_rejected, void* stream);
 
 /* The same integration as chs_integrate_batch (the fixed-step solvers of Sec.
- * Functionalities; identical results, bit for bit), run by a persistent grid (every SM filled to the kernel's occupancy) whose
+ * Functionalities; identical results, bit for bit), run by a persistent grid (every SM
+ * filled to the kernel's occupancy, as far as there are orbits) whose
  * threads take orbit indices from a work queue, one orbit after another: a
  * thread whose orbit stops early -- its t_end, early exit, escape or any other
  * freeze -- takes the next orbit at once, so orbits of uneven length leave no

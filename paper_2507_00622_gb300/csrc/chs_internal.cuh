@@ -259,4 +259,14 @@ inline cudaError_t persistent_blocks(Kernel kernel, int threads, size_t smem, un
     return cudaSuccess;
 }
 
+// Blocks of a queue launch: the persistent grid (0: unknown), but no more than the
+// ensemble has orbits for.  With idle blocks beside them the first ones to arrive take
+// the whole queue, several on one SM and none on another
+// (24,000 orbits, k = 4, 300 RK4 steps: 5.66 -> 3.78 ms; k = 3 with the LD, 38 DOP853
+// steps: 4.38 -> 2.10 ms).
+inline unsigned queue_blocks(unsigned persistent, unsigned all)
+{
+    return persistent && persistent < all ? persistent : all;
+}
+
 }  // namespace chs

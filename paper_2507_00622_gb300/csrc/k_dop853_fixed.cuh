@@ -137,7 +137,7 @@ cudaError_t fixed_sys(int k, bool ld, const StepArgs& a, const SysPar& sp, const
             static unsigned pg[kCacheDevices][2] = {};  // persistent grid per device and LD variant
             unsigned& p = pg[cache_device()][ld ? 1 : 0];
             if (!p && persistent_blocks(kern, kBlock, sm, &p) != cudaSuccess) p = 0;
-            if (p) grid = p;
+            grid = queue_blocks(p, g);
         }
         kern<<<grid, kBlock, sm, st>>>(a, sp, e, l);
     });

@@ -217,9 +217,10 @@ cudaError_t dp_pipe_k(const StepArgs& a, const SysPar& sp, const EnsPtrs& e, con
 // The pipeline pays while it fits in one wave.  us per step (one thread per orbit in
 // brackets) at 4864, 9728 and 14,592 orbits: k = 1 without the LD 8.8, 9.8 and 13.4
 // (16.1); k = 2 with the LD 9.1, 16.2 and 24.8 (29.7); k = 4 without the LD 12.6, 20.6 and
-// 30.8 (36.8); k = 4 with the LD 12.5 and 23.3 (43.7), then a second wave.  It is drained at every health check (one of its
-// iterations); at intervals below 8 steps the one-thread form runs.  A queue launch
-// of so few orbits, which hold every warp at once anyway, runs without the queue.
+// 30.8 (36.8); k = 4 with the LD 12.5 and 23.3 (43.7), then a second wave.  It is drained
+// at every health check (one of its iterations); at intervals below 8 steps the
+// one-thread form runs.  A queue launch of so few orbits, which hold every warp at
+// once anyway, runs without the queue.
 bool dp_pipe_applies(const SysPar& sp, int k, bool ld, const StepArgs& a, int64_t n)
 {
     return sp.model == CHS_HENON_HEILES && k >= 1 && k <= 4 &&

@@ -599,7 +599,7 @@ static void integ_one(const unsigned g, const StepArgs& a, const SysPar& sp, con
         unsigned& pg = pgs[cache_device()][block_slot(tb)];
         if (!pg && persistent_blocks(k_integrate<Sys, K, LD, kModeQueue>, tb, 0, &pg) != cudaSuccess)
             pg = 0;
-        k_integrate<Sys, K, LD, kModeQueue><<<pg ? pg : g, tb, 0, st>>>(a, sp, e, *ol);
+        k_integrate<Sys, K, LD, kModeQueue><<<queue_blocks(pg, g), tb, 0, st>>>(a, sp, e, *ol);
     } else if (ol) {
         k_integrate<Sys, K, LD, kModeList><<<g, tb, 0, st>>>(a, sp, e, *ol);
     } else {
