@@ -257,22 +257,76 @@ k_integrate_pipe(const StepArgs a, const SysPar sp, const EnsPtrs e, const Orbit
 // modified Gram-Schmidt of k_lyap_small in the same order, the same results.
 // 500 steps, QR every 10 on GB300, at 4864, 9728 and 14,592 orbits: 1.31, 1.84 and 2.37
 // ms, 3.07 ms with one thread per orbit; 3.12 against 3.07 ms at 19,456.
+//
+// DENSE: a section grid's FORBIDDEN cells (a quarter of it) would leave lanes empty in
+// most groups, so block b takes the OK orbits with ranks 32 b ... 32 b + 31, which every
+// block counts for itself from ic_status (a few us); blocks past the last one end.
+// A 128 x 128 section grid, 500 steps: 3.05 -> 2.35 ms.
 struct LyapSmem {
     double q[2][8][32];     // stage positions of a step
     double phi[4][16][32];  // its propagator (read by V0 and, an iteration later, V1)
     double q01[2][8][32];   // V0's unit vectors of a QR step
     int32_t bad[2][32];     // at a health check: V0's, V1's exponent sums are not finite
     int32_t live[32];       // the orbit is running
+    uint32_t ok[kLyapDenseOrbits / 32];  // DENSE: the OK orbits, a bit each
+    int32_t sums[4], pick[32];           // their number per warp's part, the block's orbits
 };
 
+// DENSE: the lane's orbit, or n; the block writes the outputs of the other orbits of
+// its own 32.
+__device__ __forceinline__ int64_t pick_orbit(LyapSmem& sm, const int64_t n, const int32_t* __restrict__ ic_status,
+                                              double* __restrict__ lambda, int32_t* __restrict__ status_out)
+{
+    constexpr int PER = (kLyapDenseOrbits / 32 + 127) / 128;
+    const int t = threadIdx.x, warp = t / 32, lane = t & 31, tiles = (int)((n + 127) / 128), words = 4 * tiles;
+#pragma unroll 8
+    for (int i = 0; i < tiles; ++i) {
+        const int64_t o = i * 128 + t;
+        const uint32_t m = __ballot_sync(0xffffffffu, o < n && ic_status[o < n ? o : 0] == CHS_ORBIT_OK);
+        if (lane == 0) sm.ok[i * 4 + warp] = m;
+    }
+    if (t < 32) sm.pick[t] = -1;
+    const int64_t own = (int64_t)blockIdx.x * 32 + lane;
+    if (own < n && ic_status[own] != CHS_ORBIT_OK) {
+        if (warp == 0) status_out[own] = ic_status[own];
+        lambda[warp * n + own] = __longlong_as_double(0x7ff8000000000000LL);
+    }
+    __syncthreads();
+    int mine = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (t * PER + i < words) mine += __popc(sm.ok[t * PER + i]);
+    int rank = mine;  // inclusive prefix over the block's threads
+#pragma unroll
+    for (int d = 1; d < 32; d *= 2) {
+        const int v = __shfl_up_sync(0xffffffffu, rank, d);
+        if (lane >= d) rank += v;
+    }
+    if (lane == 31) sm.sums[warp] = rank;
+    __syncthreads();
+    for (int i = 0; i < warp; ++i) rank += sm.sums[i];
+    rank -= mine + (int)blockIdx.x * 32;  // of the thread's first orbit, from the block's first
+    if (rank < 32 && rank + mine > 0) {
+        for (int i = 0; i < PER; ++i) {
+            if (t * PER + i >= words) break;
+            for (uint32_t m = sm.ok[t * PER + i]; m; m &= m - 1, ++rank)
+                if (rank >= 0 && rank < 32) sm.pick[rank] = (t * PER + i) * 32 + __ffs(m) - 1;
+        }
+    }
+    __syncthreads();
+    return sm.pick[lane] < 0 ? n : sm.pick[lane];
+}
+
+template <bool DENSE>
 __global__ void __launch_bounds__(128)
 k_lyap_pipe(const StepArgs a, const SysPar sp, const int64_t n, const double* __restrict__ ics,
             const int32_t* __restrict__ ic_status, double* __restrict__ lambda, int32_t* __restrict__ status_out)
 {
     __shared__ LyapSmem sm;
     const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-    const int64_t o = (int64_t)blockIdx.x * 32 + lane;
+    const int64_t o = DENSE ? pick_orbit(sm, n, ic_status, lambda, status_out) : (int64_t)blockIdx.x * 32 + lane;
     const bool valid = o < n;
+    if (DENSE && !__syncthreads_or(valid)) return;
     double x[D], w[2][D], S[2] = {0.0, 0.0};
     int32_t st = valid ? (ic_status ? ic_status[o] : CHS_ORBIT_OK) : CHS_ORBIT_FORBIDDEN;
     bool fin = true;
@@ -431,18 +485,31 @@ cudaError_t launch_integrate_pipe(const SysPar& sp, int k, bool ld, const StepAr
     return ld ? pipe_ld<true>(k, a, sp, e, ol, st) : pipe_ld<false>(k, a, sp, e, ol, st);
 }
 
-// Up to three groups of 32 orbits per SM (figures at k_lyap_pipe); health checks as
-// above.
-bool lyap_pipe_applies(const SysPar& sp, const StepArgs& a, int64_t n)
+// The DENSE form: the caller's status array may be the output array, which one block
+// would write before another has counted; then the groups stay as they lie, as they do
+// where one group per SM holds every cell.
+static bool lyap_dense(int64_t n, const int32_t* ic_status, const int32_t* status)
+{
+    const uintptr_t i = (uintptr_t)ic_status, o = (uintptr_t)status, bytes = (uintptr_t)n * sizeof(int32_t);
+    return ic_status && n > kLyapDenseFrom && n <= kLyapDenseOrbits && (i + bytes <= o || o + bytes <= i);
+}
+
+// Up to three groups of 32 orbits per SM (figures at k_lyap_pipe): 14,592 orbits, or
+// 18,432 cells of a grid, of which up to 79 % are orbits (17,000 cells, 75 % and all of
+// them OK: 2.36 and 3.13 ms, 3.08 with one thread per orbit); health checks as above.
+bool lyap_pipe_applies(const SysPar& sp, const StepArgs& a, int64_t n, const int32_t* ic_status, const int32_t* status)
 {
     return sp.model == CHS_HENON_HEILES && a.block == 0 && (a.sample_every == 0 || a.sample_every >= 16) &&
-           n <= kLyapPipeOrbits;
+           (n <= kLyapPipeOrbits || lyap_dense(n, ic_status, status));
 }
 
 cudaError_t launch_lyap_pipe(const SysPar& sp, const StepArgs& a, int64_t n, const double* ics,
                              const int32_t* ic_status, double* lambda, int32_t* status, cudaStream_t st)
 {
-    k_lyap_pipe<<<blocks_for(n, 32), 128, 0, st>>>(a, sp, n, ics, ic_status, lambda, status);
+    if (lyap_dense(n, ic_status, status))
+        k_lyap_pipe<true><<<blocks_for(n, 32), 128, 0, st>>>(a, sp, n, ics, ic_status, lambda, status);
+    else
+        k_lyap_pipe<false><<<blocks_for(n, 32), 128, 0, st>>>(a, sp, n, ics, ic_status, lambda, status);
     return cudaGetLastError();
 }
 

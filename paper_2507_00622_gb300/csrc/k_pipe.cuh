@@ -14,8 +14,8 @@ cudaError_t launch_integrate_pipe(const SysPar& sp, int k, bool ld, const StepAr
                                   const OrbitList* ol, cudaStream_t st);
 
 // The same for the Lyapunov spectrum by QR (RK4).
-constexpr int64_t kLyapPipeOrbits = 14592;
-bool lyap_pipe_applies(const SysPar& sp, const StepArgs& a, int64_t n);
+constexpr int64_t kLyapPipeOrbits = 14592, kLyapDenseFrom = 4864, kLyapDenseOrbits = 18432;
+bool lyap_pipe_applies(const SysPar& sp, const StepArgs& a, int64_t n, const int32_t* ic_status, const int32_t* status);
 cudaError_t launch_lyap_pipe(const SysPar& sp, const StepArgs& a, int64_t n, const double* ics,
                              const int32_t* ic_status, double* lambda, int32_t* status, cudaStream_t st);
 

@@ -695,7 +695,7 @@ cudaError_t launch_lyap_small(const SysPar& sp, const StepArgs& a, int64_t n, co
                               cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    if (lyap_pipe_applies(sp, a, n)) return launch_lyap_pipe(sp, a, n, ics, ic_status, lambda, status, st);
+    if (lyap_pipe_applies(sp, a, n, ic_status, status)) return launch_lyap_pipe(sp, a, n, ics, ic_status, lambda, status, st);
     const unsigned g = blocks_for(n, kSmallBlock);
     switch (sp.model) {
     case CHS_HENON_HEILES:

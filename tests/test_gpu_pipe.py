@@ -91,3 +91,27 @@ def test_pipeline_given_vectors():
     n, k = 97, 4
     w = torch.from_numpy(uniform_vectors(4, n, k, 4)).cuda()
     _same(_run(n, k, 0, 200, w_in=w, escape_r2=4.0), _run(n, k, 32, 200, w_in=w, escape_r2=4.0))
+
+
+@pytest.mark.parametrize("n", [1, 33, 4864, 4865, 7001, 14593, 18432, 18433])
+@pytest.mark.parametrize("status", ["none", "some", "few", "no orbit", "in place"])
+def test_lyapunov_pipeline_equals_one_thread_form(n, status):
+    ics = _ics(n, 3 * n)
+    rng = np.random.default_rng(n)
+    st = rng.choice([chs.ORBIT_OK, chs.ORBIT_FORBIDDEN, chs.ORBIT_ESCAPED], n, p=[0.75, 0.2, 0.05]).astype(np.int32)
+    if status == "few":
+        st[n // 50:] = chs.ORBIT_FORBIDDEN
+    elif status == "no orbit":
+        st[:] = chs.ORBIT_FORBIDDEN
+    S = chs.System(chs.HENON_HEILES, 2)
+    out = []
+    for block in (0, 32):
+        ic = None if status == "none" else torch.from_numpy(st.copy()).cuda()
+        lam = torch.full((4, n), 7.0, dtype=torch.float64, device="cuda")
+        so = ic if status == "in place" else torch.full((n,), 77, dtype=torch.int32, device="cuda")
+        chs.chs_lyapunov_spectrum(S.h, chs.params(0.01, 47, qr_every=7, sample_every=20, block_threads=block), n, ics, ic,
+                                  lam, so)
+        torch.cuda.synchronize()
+        out.append((lam.cpu().numpy(), so.cpu().numpy()))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
