@@ -1,5 +1,4 @@
-// dense.cuh -- an ensemble's running orbits dealt out evenly, for launches of a few
-// waves.
+// dense.cuh -- an ensemble's running orbits dealt out evenly over the SMs.
 //
 // With thread t on orbit t, the FORBIDDEN cells of a section grid (a quarter of it)
 // leave warps empty or partly filled, and the sub-partitions, each with its own FP64
@@ -21,68 +20,81 @@
 namespace chs {
 
 constexpr int kDenseBlocks = 152, kDenseWarps = 12, kDenseThreads = 32 * kDenseWarps;  // 168 registers a thread
-constexpr int64_t kDenseOrbits = 131072;  // largest ensemble: 128 chunks of 1024 bits
+constexpr int64_t kDenseOrbits = 1 << 20;
+constexpr size_t kDenseSmemLimit = 227 * 1024;
 
+// In dynamic shared memory: the mask of OK orbits, the number of OK orbits before each
+// chunk of 32 words (padded to whole warps), the warps' picks, the total.
 struct DenseSmem {
-    uint32_t ok[kDenseOrbits / 32];
-    int32_t before[128];  // OK orbits before each chunk of 32 words
-    int32_t pick[kDenseWarps][32];
-    int32_t total;
+    int chunks, heads;  // chunks, padded
+    uint32_t* ok;
+    int32_t *before, *pick, *total;
+    __host__ __device__ DenseSmem(void* base, const int64_t n)
+    {
+        chunks = (int)((n + 1023) / 1024);
+        heads = (chunks + 31) / 32 * 32;
+        ok = static_cast<uint32_t*>(base);
+        before = reinterpret_cast<int32_t*>(ok + 32 * chunks);
+        pick = before + heads;
+        total = pick + 32 * kDenseWarps;
+    }
+    static size_t bytes(const int64_t n)
+    {
+        const int chunks = (int)((n + 1023) / 1024);
+        return sizeof(int32_t) * (32 * chunks + (chunks + 31) / 32 * 32 + 32 * kDenseWarps + 1);
+    }
 };
 
 // The mask of OK orbits and its prefix sums; returns their number.  All threads.
-__device__ __forceinline__ int dense_scan(DenseSmem& sm, const int64_t n, const int32_t* __restrict__ status)
+__device__ __forceinline__ int dense_scan(const DenseSmem& sm, const int64_t n, const int32_t* __restrict__ status)
 {
     const int t = threadIdx.x, warp = t / 32, lane = t & 31;
-    const int words = (int)((n + 31) / 32), chunks = (words + 31) / 32;
+    const int words = (int)((n + 31) / 32);
 #pragma unroll 16
     for (int i = warp; i < words; i += kDenseWarps) {
         const int64_t o = (int64_t)i * 32 + lane;
         const uint32_t m = __ballot_sync(0xffffffffu, o < n && status[o < n ? o : 0] == CHS_ORBIT_OK);
         if (lane == 0) sm.ok[i] = m;
     }
-    if (words + t < 32 * chunks) sm.ok[words + t] = 0;
+    if (words + t < 32 * sm.chunks) sm.ok[words + t] = 0;
     __syncthreads();
-    for (int c = warp; c < 128; c += kDenseWarps) {
-        const int p = c < chunks ? __popc(sm.ok[32 * c + lane]) : 0;
+    for (int c = warp; c < sm.heads; c += kDenseWarps) {
+        const int p = c < sm.chunks ? __popc(sm.ok[32 * c + lane]) : 0;
         const int sum = __reduce_add_sync(0xffffffffu, p);
         if (lane == 0) sm.before[c] = sum;
     }
     __syncthreads();
     if (warp == 0) {
-        int v[4], sum = 0;
+        int total = 0;
+        for (int c = lane; c < sm.heads; c += 32) {
+            const int own = sm.before[c];
+            int upto = own;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            v[q] = sum;
-            sum += sm.before[4 * lane + q];
+            for (int d = 1; d < 32; d *= 2) {
+                const int u = __shfl_up_sync(0xffffffffu, upto, d);
+                if (lane >= d) upto += u;
+            }
+            sm.before[c] = total + upto - own;
+            total += __shfl_sync(0xffffffffu, upto, 31);
         }
-        int upto = sum;
-#pragma unroll
-        for (int d = 1; d < 32; d *= 2) {
-            const int u = __shfl_up_sync(0xffffffffu, upto, d);
-            if (lane >= d) upto += u;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) sm.before[4 * lane + q] = v[q] + upto - sum;
-        if (lane == 31) sm.total = upto;
+        if (lane == 0) *sm.total = total;
     }
     __syncthreads();
-    return sm.total;
+    return *sm.total;
 }
 
 // The lane's orbit of group g (a whole warp calls this), or -1.
-__device__ __forceinline__ int dense_pick(DenseSmem& sm, const int g)
+__device__ __forceinline__ int dense_pick(const DenseSmem& sm, const int g)
 {
-    const int warp = threadIdx.x / 32, lane = threadIdx.x & 31, lo = 32 * g;
+    const int lane = threadIdx.x & 31, lo = 32 * g;
+    int32_t* pick = sm.pick + (threadIdx.x - lane);
     __syncwarp();
-    sm.pick[warp][lane] = -1;
+    pick[lane] = -1;
     __syncwarp();
     int c = -1;  // the last chunk that starts at or before rank lo
-#pragma unroll
-    for (int q = 0; q < 4; ++q) c += __popc(__ballot_sync(0xffffffffu, sm.before[32 * q + lane] <= lo));
-    for (; c < 128 && sm.before[c] < lo + 32; ++c) {
-        if (c < 127 && sm.before[c + 1] == sm.before[c]) continue;  // no orbits (or past the end)
-        if (c == 127 && sm.total == sm.before[c]) break;
+    for (int q = lane; q < sm.heads; q += 32) c += __popc(__ballot_sync(0xffffffffu, sm.before[q] <= lo));
+    if (c >= sm.chunks) c = sm.chunks - 1;
+    for (; c < sm.chunks && sm.before[c] < lo + 32; ++c) {
         uint32_t m = sm.ok[32 * c + lane];
         const int p = __popc(m);
         int r = p;
@@ -93,16 +105,17 @@ __device__ __forceinline__ int dense_pick(DenseSmem& sm, const int g)
         }
         r += sm.before[c] - p - lo;  // rank of the word's first orbit within the group
         for (; m; m &= m - 1, ++r)
-            if (r >= 0 && r < 32) sm.pick[warp][r] = (32 * c + lane) * 32 + __ffs(m) - 1;
+            if (r >= 0 && r < 32) pick[r] = (32 * c + lane) * 32 + __ffs(m) - 1;
     }
     __syncwarp();
-    return sm.pick[warp][lane];
+    return pick[lane];
 }
 
 // Runs work(o) on the block's share of the OK orbits.
 template <class Work>
-__device__ __forceinline__ void dense_run(DenseSmem& sm, const EnsPtrs& e, Work work)
+__device__ __forceinline__ void dense_run(void* smem, const EnsPtrs& e, Work work)
 {
+    const DenseSmem sm(smem, e.n);
     const int groups = (dense_scan(sm, e.n, e.status) + 31) / 32;
     for (int g = threadIdx.x / 32 * kDenseBlocks + blockIdx.x; g < groups; g += kDenseWarps * kDenseBlocks) {
         const int o = dense_pick(sm, g);
@@ -126,7 +139,8 @@ __device__ __forceinline__ void store_exec(const EnsPtrs& e, const int64_t o, co
 
 // The calls it takes: a plain launch without per-orbit end steps (a warp's groups then
 // take equally long), long enough that reading the statuses (~10 us) does
-// not show.
+// not show.  Up to 2^20 orbits, whose mask is 128 KB of shared memory (reading 4 MB of
+// statuses then takes a block ~0.2 ms of at least 20).
 inline bool dense_applies(const StepArgs& a, const EnsPtrs& e, const OrbitList* ol, int64_t least_steps)
 {
     return !ol && !e.t_end && e.n <= kDenseOrbits && a.n_steps >= least_steps;
@@ -134,5 +148,22 @@ inline bool dense_applies(const StepArgs& a, const EnsPtrs& e, const OrbitList* 
 
 // The second kernel: statuses to their places.
 cudaError_t launch_dense_status(const EnsPtrs& e, cudaStream_t st);
+
+// Launches a dense kernel whose blocks need `slabs` bytes of shared memory before the
+// mask; false, with nothing launched, when they do not fit.
+template <class Kernel>
+inline bool launch_dense(Kernel kernel, const size_t slabs, const StepArgs& a, const SysPar& sp, const EnsPtrs& e,
+                         cudaStream_t st)
+{
+    const size_t bytes = slabs + DenseSmem::bytes(e.n);
+    if (bytes > kDenseSmemLimit) return false;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    kernel<<<kDenseBlocks, kDenseThreads, bytes, st>>>(a, sp, e);
+    if (cudaPeekAtLastError() == cudaSuccess) launch_dense_status(e, st);
+    return true;
+}
 
 }  // namespace chs

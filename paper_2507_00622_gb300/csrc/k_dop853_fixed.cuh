@@ -125,16 +125,15 @@ k_integrate_dp(const StepArgs a, const SysPar sp, const EnsPtrs e, const OrbitLi
 
 // The OK orbits of a few waves, dealt out evenly (dense.cuh).  Same results.
 // Section grids, k = 4 with the LD, 60 steps: 256 x 256 10.5 -> 7.63 ms; k = 4, 20 steps:
-// 130 x 140 0.93 -> 0.80, 362 x 362 5.8 -> 4.51.
+// 130 x 140 0.93 -> 0.80, 362 x 362 5.8 -> 4.51.  Slabs and mask fit up to ~530,000 cells at k = 4.
 template <class Sys, int K, bool LD>
 __global__ void __launch_bounds__(kDenseThreads, 1)
 k_integrate_dp_dense(const StepArgs a, const SysPar sp, const EnsPtrs e)
 {
     extern __shared__ double dsm[];
-    __shared__ DenseSmem sm;
     constexpr int words = (12 * Sys::NH + K * 2 * Sys::N) * kBlock;  // a warp's slab
     const dp::Slab<Sys> sl{dsm + (threadIdx.x / 32) * words + (threadIdx.x & 31)};
-    dense_run(sm, e, [&](const int64_t o) { integrate_orbit_dp<Sys, K, LD, true>(o, a, sp, e, sl); });
+    dense_run(dsm + kDenseWarps * words, e, [&](const int64_t o) { integrate_orbit_dp<Sys, K, LD, true>(o, a, sp, e, sl); });
 }
 
 // Ten steps are 0.8 ms on 65,536 cells, of which reading the statuses is 1 %.
@@ -152,15 +151,8 @@ cudaError_t fixed_sys(int k, bool ld, const StepArgs& a, const SysPar& sp, const
         auto kern = ld ? k_integrate_dp<Sys, K, true> : k_integrate_dp<Sys, K, false>;
         unsigned grid = g;
         if constexpr (K >= 1 && std::is_same<Sys, SysHenonHeiles>::value) {
-            if (dense_applies(a, e, ol, kDenseDpSteps)) {
-                auto dense = ld ? k_integrate_dp_dense<Sys, K, true> : k_integrate_dp_dense<Sys, K, false>;
-                if (cudaFuncSetAttribute(dense, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kDenseWarps * sm)) == cudaSuccess) {
-                    dense<<<kDenseBlocks, kDenseThreads, kDenseWarps * sm, st>>>(a, sp, e);
-                    if (cudaPeekAtLastError() == cudaSuccess) launch_dense_status(e, st);
-                    return;
-                }
-                cudaGetLastError();  // refused: the plain form
-            }
+            auto dense = ld ? k_integrate_dp_dense<Sys, K, true> : k_integrate_dp_dense<Sys, K, false>;
+            if (dense_applies(a, e, ol, kDenseDpSteps) && launch_dense(dense, kDenseWarps * sm, a, sp, e, st)) return;
         }
         if (l.queue) {
             static unsigned pg[kCacheDevices][2] = {};  // persistent grid per device and LD variant

@@ -371,13 +371,14 @@ k_integrate(const StepArgs a, const SysPar sp, const EnsPtrs e, const OrbitList 
 
 // The OK orbits of a few waves, dealt out evenly (dense.cuh).  Same results.
 // Section grids, k = 4 with the LD, 200 steps, before -> after: 130 x 140 1.72 -> 1.69 ms,
-// 180 x 180 2.95 -> 2.35, 256 x 256 5.37 -> 4.10, 362 x 362 9.4 -> 7.95.
+// 180 x 180 2.95 -> 2.35, 256 x 256 5.37 -> 4.10, 512 x 512 17.1 -> 15.4, 1024 x 1024 (E = 1/6)
+// 58.5 -> 56.5.
 template <class Sys, int K, bool LD>
 __global__ void __launch_bounds__(kDenseThreads, 1)
 k_integrate_dense(const StepArgs a, const SysPar sp, const EnsPtrs e)
 {
-    __shared__ DenseSmem sm;
-    dense_run(sm, e, [&](const int64_t o) { integrate_orbit<Sys, K, LD, true>(o, a, sp, e); });
+    extern __shared__ uint32_t dense_smem[];
+    dense_run(dense_smem, e, [&](const int64_t o) { integrate_orbit<Sys, K, LD, true>(o, a, sp, e); });
 }
 
 __global__ void k_dense_status(const EnsPtrs e)
@@ -637,11 +638,9 @@ static void integ_one(const unsigned g, const StepArgs& a, const SysPar& sp, con
         k_integrate<Sys, K, LD, kModeList><<<g, tb, 0, st>>>(a, sp, e, *ol);
     } else {
         if constexpr (K >= 2 && std::is_same<Sys, SysHenonHeiles>::value) {
-            if (a.block == 0 && dense_applies(a, e, ol, kDenseRk4Steps)) {
-                k_integrate_dense<Sys, K, LD><<<kDenseBlocks, kDenseThreads, 0, st>>>(a, sp, e);
-                if (cudaPeekAtLastError() == cudaSuccess) launch_dense_status(e, st);
+            if (a.block == 0 && dense_applies(a, e, ol, kDenseRk4Steps) &&
+                launch_dense(k_integrate_dense<Sys, K, LD>, 0, a, sp, e, st))
                 return;
-            }
         }
         k_integrate<Sys, K, LD, kModeAll><<<g, tb, 0, st>>>(a, sp, e, OrbitList{});
     }

@@ -1,4 +1,4 @@
-"""Plain launches on Henon-Heiles ensembles of up to 131,072 cells deal the orbits that run out to the
+"""Plain launches on Henon-Heiles ensembles of up to 2^20 cells deal the orbits that run out to the
 warps in dense groups; an explicit block size (RK4) and the work queue (DOP853) run thread t on orbit t.
 Every orbit takes the same steps, so everything is the same bit for bit: for statuses that leave full,
 ragged, empty and single-orbit groups, every way an orbit freezes, and runs split into calls."""
@@ -86,3 +86,11 @@ def test_dense_groups_health_checks_and_resume(integrator, steps, k, kw):
     _same(a, b)
     if "clock_budget" not in kw:
         _same(a, _run(30011, k, False, steps, "scattered", integrator, splits=2, **kw))
+
+
+@pytest.mark.parametrize("integrator,steps", [(chs.RK4, 100), (chs.DOP853, 10)])
+@pytest.mark.parametrize("n,k", [(300001, 2), (1 << 20, 2), ((1 << 20) + 1, 2), (1 << 20, 4)])
+def test_dense_groups_of_large_ensembles(integrator, steps, n, k):
+    kw = dict(ld_p=0.5, escape_r2=4.0, sample_every=10)
+    a, b = (_run(n, k, plain, steps, "scattered", integrator, **kw) for plain in (False, True))
+    _same(a, b)
