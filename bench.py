@@ -588,6 +588,9 @@ def run_gpu(args):
     ldi = torch.empty((2, n), dtype=torch.float64, device=dev)
     step = 0
 
+    # the plain call's form for up to 2^20 cells: k_integrate_dense and k_dense_status
+    dense = not dop and not vec_fp32 and block == 0 and rows * npy <= 1 << 20 and args.chunk >= 100
+
     def one_step(ev=None):
         nonlocal step
         prm = chs.params(DT, args.chunk, step0=step, **kw)
@@ -692,7 +695,7 @@ def run_gpu(args):
                        "grid_per_gpu": [ny, npy], "n_orbits_per_gpu": ny * npy, "dt": DT,
                        "integrator": "DOP853 (fixed step)" if dop else "RK4",
                        "steps_per_bench_step": args.chunk,
-                       "block_threads": None if dop else (block or 128),
+                       "block_threads": None if dop else 384 if dense else (block or 128),
                        "t_window": [t_window0, t_window1], "t_end_of_full_run": 1e4,
                        "deviation_vectors": f"{K_DEV} x {'fp32' if vec_fp32 else 'fp64'}",
                        "l2": "inputs larger than L2: ensemble state %.0f MB per GPU" %
@@ -702,7 +705,7 @@ def run_gpu(args):
                          "frac": achieved / peak,
                          "traffic": None if dop or block not in (0, 128) else recorded_traffic(ny, vec_fp32),
                          "kernel": "k_integrate_dp<HenonHeiles,4,LD>" if dop else
-                                   "k_integrate<HenonHeiles,4,LD>",
+                                   f"k_integrate{'_dense' if dense else ''}<HenonHeiles,4,LD>",
                          "flops_per_orbit_step": {"fp64": f64, "fp32": f32},
                          "flops_basis": "algorithmic count of the method as the oracle computes it "
                                         "(direct stage-wise RK4 on orbit, vectors and LD; FMA = 2, "
@@ -719,7 +722,7 @@ def run_gpu(args):
                        "reasons": clk["reasons"]},
             "e2e": {"value": e_orbit_steps / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d * world,
                     "d2h_bytes_per_step": d2h * world},
-            "gpu_launches": 3 * args.steps,
+            "gpu_launches": (4 if dense else 3) * args.steps,
         }
         if world == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_oracle_sample(args.chunk, args.cpu_budget,
